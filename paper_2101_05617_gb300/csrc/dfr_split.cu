@@ -19,7 +19,9 @@
 // Each JVP then runs only the imaginary half, in real arithmetic:
 //   face_tangent_kernel   traces of v, the 3 x 6 map, the hand-back;
 //   volume_tangent_kernel pointwise imaginary fluxes and sources, the DFR
-//                         sweeps (Eq. 12-14) and the augmented-operator epilogue.
+//                         sweeps (Eq. 12-14; in FP64 as block fixed point on the
+//                         integer pipe, fixed.cuh) and the augmented-operator
+//                         epilogue.
 // The imaginary parts are proportional to eps, so the tangent is propagated for
 // v itself and the final division by eps is omitted.  Results equal the plain
 // path up to rounding; no FP64 division or square root remains per JVP.
@@ -163,18 +165,13 @@ __global__ void __launch_bounds__(VolShape<NS>::THREADS, 4) volume_tangent_dev_k
 }
 
 // CTAs of a persistent volume grid: as many as fit on the GPU at once (the
-// kernel's occupancy x SMs), at most one per element tile.  Queried once per
+// kernel's occupancy x SMs), at most one per element tile, each with an even
+// share of the elements.  (6 x 60 x 60, p = 5, FP64 with the window dots: 85.3
+// us per launch; with 1 / 2 / 3 / 4 tiles a CTA in waves 94.5 / 88.8 / 86.3 /
+// 96.4 us.  6 x 30 x 30: 29.4 us, with one tile a CTA 32.6.)  Queried once per
 // kernel and device; prepare_volume_dev runs the queries of the device-driven
 // solver's kernels before its stream capture.
 constexpr int kMaxDevices = 64;
-// Element tiles per CTA of a volume grid large enough to fill the GPU three
-// times over: three tiles a CTA, the CTAs in waves.  Measured at 6 x 60 x 60,
-// p = 5 (FP64, live): 149 / 142 / 137 / 151 us per launch with 1 / 2 / 3 / 4
-// tiles a CTA and 142 us with one wave of resident CTAs taking an even share
-// (the four CTAs of an SM then run their load and compute phases in step).
-// Smaller grids take one wave of resident CTAs with an even share each.
-constexpr int kVolTilesPerCta = 3;
-
 template <typename T, int NS, bool W3, bool DEV>
 int volume_ctas(int device, long long tiles) {
   static int fit[kMaxDevices] = {};
@@ -190,7 +187,6 @@ int volume_ctas(int device, long long tiles) {
     if (e != cudaSuccess || nb < 1) return -1;
     fit[device] = nb * sms;
   }
-  if (tiles >= (long long)kVolTilesPerCta * fit[device]) return (int)((tiles + kVolTilesPerCta - 1) / kVolTilesPerCta);
   return (int)std::min<long long>(std::max<long long>(tiles, 1), fit[device]);
 }
 

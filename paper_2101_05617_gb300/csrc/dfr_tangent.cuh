@@ -8,6 +8,7 @@
 #include "check.cuh"
 #include "convert.cuh"
 #include "dfr_device.cuh"
+#include "fixed.cuh"
 #include "swepi_internal.h"
 
 namespace swepi {
@@ -120,16 +121,20 @@ struct VolSmem {
   T sF[EPB][2][3][NS * NS];   // fluxes along xi^1 and xi^2
   T sB[EPB][4][3][NS];        // interface fluxes of the four edges
   T sD[NS][NS + 3];           // derivative matrix, padded rows: distinct banks per k
+  unsigned sE[2][EPB][2];     // FP64: largest magnitude keys of the elements' fluxes (mass, momentum), by tile parity
 };
 
-// derivative matrix pre-multiplied by -(2/dx) * scale (Eq. 14 and the
-// augmented operator's dt) into shared memory: each output is then one chain
-// of fused multiply-adds started from scale * source
+// derivative matrix into shared memory: in FP32 pre-multiplied by -(2/dx) *
+// scale (Eq. 14 and the augmented operator's dt), so that each output is one
+// chain of fused multiply-adds started from scale * source; in FP64 the packed
+// integer matrix of the block fixed-point sweeps
 template <typename T, int NS, int EPB, int BLOCK>
 __device__ __forceinline__ void tile_dmat(const TanVolArgs<T>& a, const DfrConst& dc, VolSmem<T, NS, EPB>& sm) {
   const double dscale = -dc.two_over_dx * a.ep.scale;
-  for (int t = threadIdx.x; t < NS * (NS + 2); t += BLOCK)
-    sm.sD[t / (NS + 2)][t % (NS + 2)] = from_f64<T>(dscale * dc.D[t / (NS + 2)][t % (NS + 2)]);
+  for (int t = threadIdx.x; t < NS * (NS + 2); t += BLOCK) {
+    if constexpr (sizeof(T) == 4) sm.sD[t / (NS + 2)][t % (NS + 2)] = from_f64<T>(dscale * dc.D[t / (NS + 2)][t % (NS + 2)]);
+    else sm.sD[t / (NS + 2)][t % (NS + 2)] = dc.Dq[t / (NS + 2)][t % (NS + 2)];
+  }
 }
 
 // interface fluxes of the four edges of the elements eb .. eb + EPB - 1 (those
@@ -165,6 +170,153 @@ __device__ __forceinline__ void tile_fluxes(const TanVolArgs<T>& a, VolSmem<T, N
   sm.sF[le][1][0][node] = v2;
   sm.sF[le][1][1][node] = F12;
   sm.sF[le][1][2][node] = F22;
+}
+
+// ---- FP64: the DFR sweeps in block fixed point (fixed.cuh)
+// The 6 (N_s + 2) multiply-adds per node of the two sweeps are over half of
+// the kernel's FP64 operations, and the kernel is bound by the FP64 pipe.  Every line
+// of an element shares a scale, so the element's fluxes (mass and momentum
+// apart: their units differ) are packed once, seven conversions a node, and
+// the sweeps run as integer multiply-adds.  An element that the format cannot
+// hold keeps FP64 values in the same arrays and takes the FP64 chain.
+// 6 x 60 x 60, p = 5, with the augmented operator and the window dots: 134 ->
+// 85 us (FP64 pipe 87 -> 66 %: ~41 FP64 instructions a node are left of 83, the
+// point fluxes 15, the b columns 12, the window dots 6); the product alone 129
+// -> 79 us with its face kernel, 6 x 90 x 90, p = 6: 395 -> 217 us.  Relative
+// error against a 64-bit reference unchanged (3.5e-15, the reference's own).
+
+// what one node brings to its element: its fluxes, and its share of the
+// element's 12 N_s interface fluxes
+template <int NS>
+struct FxPoint {
+  static constexpr int EC = (12 + NS - 1) / NS;   // interface values per thread
+  double v1, v2, F11, F12, F22;
+  double e[EC];
+};
+
+// m0, m1: largest magnitude keys of the mass and the momentum fluxes
+template <int NS>
+__device__ __forceinline__ void fx_edges(const double* __restrict__ fb, long long elem, int node, FxPoint<NS>& pt,
+                                         unsigned& m0, unsigned& m1) {
+  constexpr int NN = NS * NS;
+#pragma unroll
+  for (int i = 0; i < FxPoint<NS>::EC; ++i) {
+    const int r = node + i * NN;
+    pt.e[i] = 0.0;
+    if (r < 12 * NS) {
+      pt.e[i] = fb[elem * 12 * NS + r];
+      const unsigned m = fx_key(pt.e[i]);
+      if ((r / NS) % 3 == 0) m0 = max(m0, m);
+      else m1 = max(m1, m);
+    }
+  }
+  m0 = max(m0, max(fx_key(pt.v1), fx_key(pt.v2)));
+  m1 = max(m1, max(fx_key(pt.F11), max(fx_key(pt.F12), fx_key(pt.F22))));
+}
+
+// the node's values into the tile's arrays sF [2][3][NN], sB [12 NS] of its
+// element: packed where the element's keys M0, M1 allow (fixed), else as they are
+template <int NS>
+__device__ __forceinline__ void fx_store(double (*sF)[3][NS * NS], double* sB, int node, const FxPoint<NS>& pt,
+                                         bool fixed, unsigned M0, unsigned M1) {
+  constexpr int NN = NS * NS;
+  const int E0 = fx_exp(M0), E1 = fx_exp(M1);
+  double v1 = pt.v1, v2 = pt.v2, F11 = pt.F11, F12 = pt.F12, F22 = pt.F22;
+  if (fixed) {
+    v1 = fx_pack(v1, E0);
+    v2 = fx_pack(v2, E0);
+    F11 = fx_pack(F11, E1);
+    F12 = fx_pack(F12, E1);
+    F22 = fx_pack(F22, E1);
+  }
+  sF[0][0][node] = v1;
+  sF[0][1][node] = F11;
+  sF[0][2][node] = F12;
+  sF[1][0][node] = v2;
+  sF[1][1][node] = F12;
+  sF[1][2][node] = F22;
+#pragma unroll
+  for (int i = 0; i < FxPoint<NS>::EC; ++i) {
+    const int r = node + i * NN;
+    if (r < 12 * NS) sB[r] = fixed ? fx_pack(pt.e[i], (r / NS) % 3 == 0 ? E0 : E1) : pt.e[i];
+  }
+}
+
+// a scale the packed sweeps can be multiplied by through its exponent field
+__device__ __forceinline__ bool fx_scale_usable(double s) {
+  const int e = (__double2hiint(s) >> 20) & 0x7ff;
+  return e >= 823 && e <= 1223;
+}
+
+// the two sweeps of node (k2, k1): res[mu] = dscale * (D-row k1 along xi^1 +
+// D-row k2 along xi^2) + add[mu] (add[0] is zero).  Da, Db: the packed rows in
+// shared memory (each entry read once for the three variables: rows held in
+// registers spilled); sB [4][3][NS].  The packed sum is converted once (one
+// FP64 instruction) and scaled by dscale with the blocks' exponents added to
+// its exponent field.
+template <int NS>
+__device__ __forceinline__ void fx_sweep(const double (*sF)[3][NS * NS], const double* sB, int k1, int k2,
+                                         const double* Da, const double* Db, const DfrConst& dc,
+                                         double dscale, bool fixed, unsigned M0, unsigned M1, double add1, double add2,
+                                         double res[3]) {
+  if (fixed) {
+    FxAcc a[3];
+#pragma unroll
+    for (int l = 0; l < NS + 2; ++l) {
+      const double m = Da[l];
+#pragma unroll
+      for (int mu = 0; mu < 3; ++mu)
+        fx_mac(a[mu], l == 0 ? sB[mu * NS + k2] : (l == NS + 1 ? sB[(3 + mu) * NS + k2] : sF[0][mu][k2 * NS + l - 1]), m);
+    }
+#pragma unroll
+    for (int l = 0; l < NS + 2; ++l) {
+      const double m = Db[l];
+#pragma unroll
+      for (int mu = 0; mu < 3; ++mu)
+        fx_mac(a[mu], l == 0 ? sB[(6 + mu) * NS + k1] : (l == NS + 1 ? sB[(9 + mu) * NS + k1] : sF[1][mu][(l - 1) * NS + k1]), m);
+    }
+    const int sh = __double2hiint(dscale), sl = __double2loint(dscale);
+#pragma unroll
+    for (int mu = 0; mu < 3; ++mu) {
+      const int k = fx_exp(mu == 0 ? M0 : M1) + dc.dq_exp;
+      const double sc = __hiloint2double(sh + k * 1048576, sl);
+      const double s = fx_sum(a[mu]);
+      res[mu] = mu == 0 ? s * sc : fma(s, sc, mu == 1 ? add1 : add2);
+    }
+    return;
+  }
+#pragma unroll 1
+  for (int mu = 0; mu < 3; ++mu) {
+    double c = mu == 0 ? 0.0 : (mu == 1 ? add1 : add2);
+    c = fma(dscale * dc.D[k1][0], sB[(0 * 3 + mu) * NS + k2], c);
+    c = fma(dscale * dc.D[k1][NS + 1], sB[(1 * 3 + mu) * NS + k2], c);
+#pragma unroll 1
+    for (int l = 0; l < NS; ++l) c = fma(dscale * dc.D[k1][l + 1], sF[0][mu][k2 * NS + l], c);
+    c = fma(dscale * dc.D[k2][0], sB[(2 * 3 + mu) * NS + k1], c);
+    c = fma(dscale * dc.D[k2][NS + 1], sB[(3 * 3 + mu) * NS + k1], c);
+#pragma unroll 1
+    for (int l = 0; l < NS; ++l) c = fma(dscale * dc.D[k2][l + 1], sF[1][mu][l * NS + k1], c);
+    if (mu == 0) res[0] = c;
+    else if (mu == 1) res[1] = c;
+    else res[2] = c;
+  }
+}
+
+// pointwise imaginary fluxes of node idx into pt, the sources S^1, S^2 returned
+template <int NS>
+__device__ __forceinline__ void tan_fluxes(const TanVolArgs<double>& a, long long idx, FxPoint<NS>& pt, double& S1,
+                                           double& S2) {
+  const long long N = a.nodes;
+  const double v0 = __ldg(a.v + idx), v1 = __ldg(a.v + idx + N), v2 = __ldg(a.v + idx + 2 * N);
+  const double* ln = a.ln + idx;
+  const double u1 = ln[LN_U1 * N], u2 = ln[LN_U2 * N];
+  pt.F11 = fma(2.0 * u1, v1, ln[LN_A11 * N] * v0);
+  pt.F12 = fma(u2, v1, fma(u1, v2, ln[LN_A12 * N] * v0));
+  pt.F22 = fma(2.0 * u2, v2, ln[LN_A22 * N] * v0);
+  S1 = fma(ln[LN_S11 * N], v1, fma(ln[LN_S12 * N], v2, ln[LN_S10 * N] * v0));
+  S2 = fma(ln[LN_S21 * N], v1, fma(ln[LN_S22 * N], v2, ln[LN_S20 * N] * v0));
+  pt.v1 = v1;
+  pt.v2 = v2;
 }
 
 // the two DFR sweeps of one node (rows Da, Db of the scaled derivative
@@ -220,32 +372,39 @@ template <typename T, int NS, int EPB, int BLOCK = EPB * NS * NS, bool W3 = fals
 __device__ __forceinline__ void volume_tangent_body(const TanVolArgs<T>& a, const DfrConst& dc, unsigned int blk,
                                                     unsigned int nblk, VolSmem<T, NS, EPB>& sm) {
   constexpr int NN = NS * NS;
+  constexpr bool F32 = sizeof(T) == 4;
   static_assert(EPB * NN <= BLOCK, "block too small for the element tile");
+  static_assert(!F32, "the batched kernels run in FP64");
   tile_dmat<T, NS, EPB, BLOCK>(a, dc, sm);
+  for (int t = threadIdx.x; t < 2 * EPB; t += BLOCK) sm.sE[0][t >> 1][t & 1] = 0u;
   const int le = threadIdx.x / NN, node = threadIdx.x % NN;
-  const long long eb = (long long)blk * EPB;
-  const long long elem = eb + le;
+  const long long elem = (long long)blk * EPB + le;
   const bool active = threadIdx.x < EPB * NN && elem < a.nelem;
   const int k2 = node / NS, k1 = node % NS;
   const long long idx = elem * NN + node;
-  tile_edges<T, NS, EPB, BLOCK>(a, sm, eb, a.nelem);
-  T S1 = T(0), S2 = T(0);
-  if (active) tile_fluxes<T, NS, EPB>(a, sm, le, node, idx, S1, S2);
-  constexpr bool F32 = sizeof(T) == 4;
-  __shared__ float coef32[MAX_NB];
-  tile_coef32<T>(a.ep, coef32);
+  const double dscale = -dc.two_over_dx * a.ep.scale;
+  FxPoint<NS> pt;
+  double S1 = 0.0, S2 = 0.0;
+  unsigned m0 = 0u, m1 = 0u;
+  if (active) {
+    tan_fluxes<NS>(a, idx, pt, S1, S2);
+    fx_edges<NS>(a.fb, elem, node, pt, m0, m1);
+  }
+  __syncthreads();
+  fx_block_max<NN, EPB, BLOCK>(sm.sE[0], le, m0, m1);
+  __syncthreads();
+  bool fixed = false;
+  if (active) {
+    m0 = sm.sE[0][le][0];
+    m1 = sm.sE[0][le][1];
+    fixed = fx_usable(m0) && fx_usable(m1) && fx_scale_usable(dscale);
+    fx_store<NS>(sm.sF[le], &sm.sB[le][0][0][0], node, pt, fixed, m0, m1);
+  }
   __syncthreads();
   double res[3] = {0.0, 0.0, 0.0};
   if (active) {
-    // this thread's rows of the derivative matrix, from shared memory into registers
-    // (a per-thread row index into the constant bank would serialise the warp)
-    T Da[NS + 2], Db[NS + 2];
-#pragma unroll
-    for (int n = 0; n < NS + 2; ++n) {
-      Da[n] = sm.sD[k1][n];
-      Db[n] = sm.sD[k2][n];
-    }
-    tile_sweep<T, NS, EPB>(a, sm, le, k1, k2, idx, Da, Db, from_f64<T>(a.ep.scale), S1, S2, coef32, res);
+    fx_sweep<NS>(sm.sF[le], &sm.sB[le][0][0][0], k1, k2, sm.sD[k1], sm.sD[k2], dc, dscale, fixed, m0, m1, a.ep.scale * S1,
+                 a.ep.scale * S2, res);
   }
   volume_epilogue<BLOCK, true, W3, !F32, F32>(a.ep, active, idx, a.nodes, res, a.out, blk, nblk);
 }
@@ -267,31 +426,69 @@ __device__ __forceinline__ void volume_tangent_persistent(const TanVolArgs<T>& a
   __shared__ float coef32[MAX_NB];
   if (!F32) epilogue_coefs(a.ep, coef);
   tile_coef32<T>(a.ep, coef32);
+  if (!F32)
+    for (int t = threadIdx.x; t < 2 * EPB; t += BLOCK) sm.sE[0][t >> 1][t & 1] = 0u;
   __syncthreads();
   const int le = threadIdx.x / NN, node = threadIdx.x % NN;
   const int k2 = node / NS, k1 = node % NS;
   const bool lane_on = threadIdx.x < EPB * NN;
-  T Da[NS + 2], Db[NS + 2];
-#pragma unroll
-  for (int n = 0; n < NS + 2; ++n) {
-    Da[n] = lane_on ? sm.sD[k1][n] : T(0);
-    Db[n] = lane_on ? sm.sD[k2][n] : T(0);
-  }
-  const T sc = from_f64<T>(a.ep.scale);
   double da = 0.0, db = 0.0, dcc = 0.0, dab = 0.0, dbc = 0.0;
-  for (long long eb = e0; eb < e1; eb += EPB) {
-    const long long elem = eb + le;
-    const bool active = lane_on && elem < e1;
-    const long long idx = elem * NN + node;
-    __syncthreads();   // the previous tile's readers are done with sF and sB
-    tile_edges<T, NS, EPB, BLOCK>(a, sm, eb, e1);
-    T S1 = T(0), S2 = T(0);
-    if (active) tile_fluxes<T, NS, EPB>(a, sm, le, node, idx, S1, S2);
-    __syncthreads();
-    if (active) {
-      double res[3];
-      tile_sweep<T, NS, EPB>(a, sm, le, k1, k2, idx, Da, Db, sc, S1, S2, coef32, res);
-      epilogue_node<W3, !F32, F32>(a.ep, coef, idx, a.nodes, res, a.out, da, db, dcc, dab, dbc);
+  if constexpr (F32) {
+    T Da[NS + 2], Db[NS + 2];
+#pragma unroll
+    for (int n = 0; n < NS + 2; ++n) {
+      Da[n] = lane_on ? sm.sD[k1][n] : T(0);
+      Db[n] = lane_on ? sm.sD[k2][n] : T(0);
+    }
+    const T sc = from_f64<T>(a.ep.scale);
+    for (long long eb = e0; eb < e1; eb += EPB) {
+      const long long elem = eb + le;
+      const bool active = lane_on && elem < e1;
+      const long long idx = elem * NN + node;
+      __syncthreads();   // the previous tile's readers are done with sF and sB
+      tile_edges<T, NS, EPB, BLOCK>(a, sm, eb, e1);
+      T S1 = T(0), S2 = T(0);
+      if (active) tile_fluxes<T, NS, EPB>(a, sm, le, node, idx, S1, S2);
+      __syncthreads();
+      if (active) {
+        double res[3];
+        tile_sweep<T, NS, EPB>(a, sm, le, k1, k2, idx, Da, Db, sc, S1, S2, coef32, res);
+        epilogue_node<W3, !F32, F32>(a.ep, coef, idx, a.nodes, res, a.out, da, db, dcc, dab, dbc);
+      }
+    }
+  } else {
+    const double dscale = -dc.two_over_dx * a.ep.scale;
+    const bool scale_ok = fx_scale_usable(dscale);
+    int par = 0;
+    for (long long eb = e0; eb < e1; eb += EPB, par ^= 1) {
+      const long long elem = eb + le;
+      const bool active = lane_on && elem < e1;
+      const long long idx = elem * NN + node;
+      FxPoint<NS> pt;
+      double S1 = 0.0, S2 = 0.0;
+      unsigned m0 = 0u, m1 = 0u;
+      if (active) {
+        tan_fluxes<NS>(a, idx, pt, S1, S2);
+        fx_edges<NS>(a.fb, elem, node, pt, m0, m1);
+      }
+      // this parity's keys were zeroed before the previous tile's last barrier
+      fx_block_max<NN, EPB, BLOCK>(sm.sE[par], le, m0, m1);
+      __syncthreads();   // the keys are complete; the previous tile's readers are done with sF and sB
+      bool fixed = false;
+      if (active) {
+        m0 = sm.sE[par][le][0];
+        m1 = sm.sE[par][le][1];
+        fixed = scale_ok && fx_usable(m0) && fx_usable(m1);
+        fx_store<NS>(sm.sF[le], &sm.sB[le][0][0][0], node, pt, fixed, m0, m1);
+      }
+      for (int t = threadIdx.x; t < 2 * EPB; t += BLOCK) sm.sE[par ^ 1][t >> 1][t & 1] = 0u;
+      __syncthreads();
+      if (active) {
+        double res[3];
+        fx_sweep<NS>(sm.sF[le], &sm.sB[le][0][0][0], k1, k2, sm.sD[k1], sm.sD[k2], dc, dscale, fixed, m0, m1, a.ep.scale * S1,
+                     a.ep.scale * S2, res);
+        epilogue_node<W3, !F32, F32>(a.ep, coef, idx, a.nodes, res, a.out, da, db, dcc, dab, dbc);
+      }
     }
   }
   __shared__ double sred[(F32 ? 5 : 3) * BLOCK];

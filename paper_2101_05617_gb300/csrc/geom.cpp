@@ -46,6 +46,40 @@ void gauss_legendre(int N, std::vector<double>& x, std::vector<double>& w) {
   }
 }
 
+// Fixed coefficients as integers for the block fixed-point sums (fixed.cuh):
+// c = X 2^(e - 58) with 2^e above the largest of them, X rounded to nearest,
+// X = h 2^29 + l with |l| <= 2^28; h and l are stored as the high and low word
+// of a double.  A sum over values f = Y 2^(E - 1022 - 58) (E the block's biased
+// exponent) then is sum X Y = S 2^58 with S in units of 2^(E - 1080 + e).
+int pack_exponent(double largest) {
+  int e = 0;
+  std::frexp(largest, &e);   // largest = f 2^e, f in [1/2, 1)
+  return e;
+}
+double pack_coefficient(double c, int e) {
+  const long long X = std::llrint(std::ldexp(c, 58 - e));
+  const long long h = (X + (1ll << 28)) >> 29, l = X - h * (1ll << 29);
+  const uint64_t bits = ((uint64_t)(uint32_t)(int32_t)h << 32) | (uint32_t)(int32_t)l;
+  double d;
+  std::memcpy(&d, &bits, sizeof(bits));
+  return d;
+}
+void pack_operators(DfrConst& dc, int ns) {
+  double D = 0.0, l = 0.0;
+  for (int k = 0; k < ns; ++k) {
+    for (int n = 0; n < ns + 2; ++n) D = std::fmax(D, std::fabs(dc.D[k][n]));
+    l = std::fmax(l, std::fmax(std::fabs(dc.lm[k]), std::fabs(dc.lp[k])));
+  }
+  const int De = pack_exponent(D), le = pack_exponent(l);
+  dc.dq_exp = De - 1080;
+  dc.lq_exp = le - 1080;
+  for (int k = 0; k < ns; ++k) {
+    for (int n = 0; n < ns + 2; ++n) dc.Dq[k][n] = pack_coefficient(dc.D[k][n], De);
+    dc.lmq[k] = pack_coefficient(dc.lm[k], le);
+    dc.lpq[k] = pack_coefficient(dc.lp[k], le);
+  }
+}
+
 // Barycentric weights of a node set.
 std::vector<double> bary_weights(const std::vector<double>& z) {
   int n = (int)z.size();
@@ -261,6 +295,7 @@ int build_tables(Ctx& c) {
   c.Dg = (ns == 1) ? std::vector<double>(1, 0.0) : bary_diff(c.xi);
   for (int k = 0; k < ns; ++k)
     for (int l = 0; l < ns; ++l) c.dc.Dg[k][l] = c.Dg[k * ns + l];
+  pack_operators(c.dc, ns);
   c.dc.two_over_dx = 2.0 / c.dx;
   c.dc.gravity = c.prm.gravity;
 

@@ -71,8 +71,12 @@ struct FaceLine {
 // Small DFR constants passed by value to the kernels.
 struct DfrConst {
   double D[MAX_NS][MAX_NS + 2];   // l~'_n(xi_k), Eq. (12)-(13)
+  double Dq[MAX_NS][MAX_NS + 2];  // the same as packed integers of the block fixed-point sweeps (fixed.cuh)
+  int dq_exp;                     // a packed sweep of a block with exponent E is in units of 2^(E + dq_exp)
   double Dg[MAX_NS][MAX_NS];      // l'_l(xi_k) on the solution points (collocation derivative)
   double lm[MAX_NS], lp[MAX_NS];  // l_k(-1), l_k(+1), Eq. (8)
+  double lmq[MAX_NS], lpq[MAX_NS];   // the same packed
+  int lq_exp;                     // a packed trace of a block with exponent E is in units of 2^(E + lq_exp)
   float lm32[MAX_NS], lp32[MAX_NS];  // the same rounded to FP32 (complex64-bulk form)
   double two_over_dx;             // Eq. (6)
   double gravity;
