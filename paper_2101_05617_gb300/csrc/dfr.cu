@@ -28,6 +28,7 @@
 
 #include "check.cuh"
 #include "dfr_device.cuh"
+#include "dfr_tangent.cuh"
 #include "swepi_internal.h"
 
 namespace swepi {
@@ -96,29 +97,26 @@ struct VolArgs {
   AugEpilogue ep;
 };
 
+// The two sweeps are 48 of the ~75 (right-hand side) to ~120 (product) FP64
+// instructions a node at N_s = 6, and the FP64 pipe bounds the kernel: they run
+// as block fixed point on the integer pipe (fixed.cuh, dfr_tangent.cuh).
 template <typename T, int NS, bool W3 = false>
 __global__ void __launch_bounds__(VolShape<NS>::THREADS) volume_kernel(VolArgs a, DfrConst dc) {
   constexpr int EPB = VolShape<NS>::EPB;
   constexpr int NN = NS * NS;
   if (a.ep.skip && *a.ep.skip) return;
-  __shared__ double sF[EPB][2][3][NN];       // [dir][mu][k2*NS+k1]
-  __shared__ double sB[EPB][4][3][NS];       // face fluxes [edge][mu][pt]
-  __shared__ double sD[NS][NS + 3];          // padded rows: distinct banks per k
-  for (int t = threadIdx.x; t < NS * (NS + 2); t += blockDim.x) sD[t / (NS + 2)][t % (NS + 2)] = dc.D[t / (NS + 2)][t % (NS + 2)];
+  __shared__ VolSmem<double, NS, EPB> sm;
+  for (int t = threadIdx.x; t < NS * (NS + 2); t += blockDim.x) sm.sD[t / (NS + 2)][t % (NS + 2)] = dc.Dq[t / (NS + 2)][t % (NS + 2)];
+  for (int t = threadIdx.x; t < 2 * EPB; t += blockDim.x) sm.sE[0][t >> 1][t & 1] = 0u;
   const int le = threadIdx.x / NN, node = threadIdx.x % NN;
   const long long elem = (long long)blockIdx.x * EPB + le;
   const bool active = elem < a.nelem;
   const int k2 = node / NS, k1 = node % NS;
   const long long idx = elem * NN + node;
 
-  // face fluxes of this block's elements
-  for (int t = threadIdx.x; t < EPB * 12 * NS; t += blockDim.x) {
-    int e = t / (12 * NS), r = t % (12 * NS);
-    long long ge = (long long)blockIdx.x * EPB + e;
-    (&sB[e][0][0][0])[r] = (ge < a.nelem) ? a.fb[ge * 12 * NS + r] : 0.0;
-  }
-
-  T S[3];
+  FxPoint<NS> pt;
+  double S1 = 0.0, S2 = 0.0;
+  unsigned m0 = 0u, m1 = 0u;
   if (active) {
     const long long N = a.nodes;
     T q0 = load_state<T>(a.q, a.v, a.eps, idx);
@@ -128,52 +126,41 @@ __global__ void __launch_bounds__(VolShape<NS>::THREADS) volume_kernel(VolArgs a
     T r = cs_rcp(q0);
     T u1 = q1 * r, u2 = q2 * r;
     T q0sq = q0 * q0;
-    T F11 = q1 * u1 + nc[NC_C11 * N] * q0sq;     // sqrt(g) T^{mu nu}, Eq. (136)
-    T F12 = q1 * u2 + nc[NC_C12 * N] * q0sq;
-    T F22 = q2 * u2 + nc[NC_C22 * N] * q0sq;
     T q1u1 = q1 * u1, q1u2 = q1 * u2, q2u2 = q2 * u2;
     // sources of Eq. (2): Coriolis, metric (Gamma^i_jk), topography
-    S[0] = mk(0.0, 0.0, (T*)nullptr);
-    S[1] = (nc[NC_K11 * N] * q1 + nc[NC_K12 * N] * q2) - (nc[NC_G1A * N] * q1u1 + nc[NC_G1B * N] * q1u2) +
-           nc[NC_B1 * N] * q0;
-    S[2] = (nc[NC_K21 * N] * q1 + nc[NC_K22 * N] * q2) - (nc[NC_G2A * N] * q1u2 + nc[NC_G2B * N] * q2u2) +
-           nc[NC_B2 * N] * q0;
-    sF[le][0][0][node] = part(q1);
-    sF[le][0][1][node] = part(F11);
-    sF[le][0][2][node] = part(F12);
-    sF[le][1][0][node] = part(q2);
-    sF[le][1][1][node] = part(F12);
-    sF[le][1][2][node] = part(F22);
+    S1 = part((nc[NC_K11 * N] * q1 + nc[NC_K12 * N] * q2) - (nc[NC_G1A * N] * q1u1 + nc[NC_G1B * N] * q1u2) +
+              nc[NC_B1 * N] * q0);
+    S2 = part((nc[NC_K21 * N] * q1 + nc[NC_K22 * N] * q2) - (nc[NC_G2A * N] * q1u2 + nc[NC_G2B * N] * q2u2) +
+              nc[NC_B2 * N] * q0);
+    pt.v1 = part(q1);
+    pt.v2 = part(q2);
+    pt.F11 = part(q1u1 + nc[NC_C11 * N] * q0sq);     // sqrt(g) T^{mu nu}, Eq. (136)
+    pt.F12 = part(q1u2 + nc[NC_C12 * N] * q0sq);
+    pt.F22 = part(q2u2 + nc[NC_C22 * N] * q0sq);
+    fx_edges<NS>(a.fb, elem, node, pt, m0, m1);
+  }
+  __syncthreads();
+  fx_block_max<NN, EPB, VolShape<NS>::THREADS>(sm.sE[0], le, m0, m1);
+  __syncthreads();
+  const double dscale = -dc.two_over_dx;
+  bool fixed = false;
+  if (active) {
+    m0 = sm.sE[0][le][0];
+    m1 = sm.sE[0][le][1];
+    fixed = fx_usable(m0) && fx_usable(m1) && fx_scale_usable(dscale);
+    fx_store<NS>(sm.sF[le], &sm.sB[le][0][0][0], node, pt, fixed, m0, m1);
   }
   __syncthreads();
 
   // DFR sweeps: extended flux [F(-1), f_1..f_NS, F(+1)] per line (Eq. 11-14)
-  // this thread's rows of the derivative matrix, from shared memory into registers
-  // (a per-thread row index into the constant bank would serialise the warp)
   double res[3] = {0.0, 0.0, 0.0};
-  double Da[NS + 2], Db[NS + 2];
-#pragma unroll
-  for (int n = 0; n < NS + 2; ++n) {
-    Da[n] = sD[k1][n];
-    Db[n] = sD[k2][n];
-  }
   if (active) {
+    fx_sweep<NS>(sm.sF[le], &sm.sB[le][0][0][0], k1, k2, sm.sD[k1], sm.sD[k2], dc, dscale, fixed, m0, m1, S1, S2, res);
+    if (a.v) {
+      const double sc = 1.0 / a.eps;
 #pragma unroll
-    for (int mu = 0; mu < 3; ++mu) {
-      double d1 = Da[0] * sB[le][0][mu][k2] + Da[NS + 1] * sB[le][1][mu][k2];
-      double d2 = Db[0] * sB[le][2][mu][k1] + Db[NS + 1] * sB[le][3][mu][k1];
-#pragma unroll
-      for (int l = 0; l < NS; ++l) {
-        d1 = fma(Da[l + 1], sF[le][0][mu][k2 * NS + l], d1);
-        d2 = fma(Db[l + 1], sF[le][1][mu][l * NS + k1], d2);
-      }
-      res[mu] = -dc.two_over_dx * (d1 + d2) + part(S[mu]);
+      for (int mu = 0; mu < 3; ++mu) res[mu] *= sc;
     }
-  }
-  if (active) {
-    const double sc = a.v ? 1.0 / a.eps : 1.0;
-#pragma unroll
-    for (int mu = 0; mu < 3; ++mu) res[mu] *= sc;
   }
   volume_epilogue<VolShape<NS>::THREADS, false, W3>(a.ep, active, idx, a.nodes, res, a.out, blockIdx.x, gridDim.x);
 }
