@@ -6,6 +6,7 @@
 
 #include <cuda_runtime.h>
 
+#include "fixed.cuh"
 #include "swepi_internal.h"
 
 namespace swepi {
@@ -55,33 +56,37 @@ __device__ __forceinline__ T load_state(const double* __restrict__ q, const doub
 }
 
 // ---------------------------------------------------------------- AUSM
-// basic AUSM splittings (reading of App. D Eq. 138-139; [41] Eq. 6 and 8)
-template <typename T>
-__device__ __forceinline__ void ausm_side(const T q[3], int d, double ad, double p1, double p2, T& M, T A[3], T P[3]) {
-  T a = cs_sqrt(ad * q[0]);                       // a^d = sqrt(h^dd g_r H), App. E
-  T u = cs_div(q[d], q[0]);                       // u^d
-  M = cs_div(u, a);                               // Froude number
-  A[0] = a * q[0];                                // A^{mu d} = a q^mu
-  A[1] = a * q[1];
-  A[2] = a * q[2];
-  T q0sq = q[0] * q[0];
-  P[0] = 0.0 * q[0];
-  P[1] = p1 * q0sq;                               // P^{mu d} = g_r h^{mu d} (q^0)^2 / (2 sqrt g)
-  P[2] = p2 * q0sq;
+// FP64 divisions and square roots are sequences of many FP64 instructions, so
+// each side takes one square root and the fewest reciprocals (a^d and u^d/a^d;
+// the complex step shares 1/q^0 and 1/a^d between its halves).
+// a^d = sqrt(h^dd g_r H) (App. E) and the Froude number M = u^d / a^d
+__device__ __forceinline__ void speed_mach(double q0, double qd, double ad, double& a, double& M) {
+  a = sqrt(ad * q0);
+  M = qd / (q0 * a);
+}
+__device__ __forceinline__ void speed_mach(cs q0, cs qd, double ad, cs& a, cs& M) {
+  const double s = sqrt(ad * q0.re), is = 1.0 / s, r = 1.0 / q0.re;
+  a = {s, (0.5 * ad) * q0.im * is};
+  const double u = qd.re * r, ui = (qd.im - u * q0.im) * r;
+  const double m = u * is;
+  M = {m, (ui - m * a.im) * is};
 }
 
+// AUSM interface flux, basic splittings (reading of App. D Eq. 138-139; [41]
+// Eq. 6 and 8): flux^mu = M_{1/2} a q^mu (upwind side) + beta+ P_L + beta- P_R
+// with P^{mu d} = g_r h^{mu d} (q^0)^2 / (2 sqrt g), zero for mu = 0
 template <typename T>
 __device__ __forceinline__ void ausm_flux(const T qL[3], const T qR[3], int d, double ad, double p1, double p2,
                                           T flux[3]) {
-  T ML, MR, AL[3], AR[3], PL[3], PR[3];
-  ausm_side(qL, d, ad, p1, p2, ML, AL, PL);
-  ausm_side(qR, d, ad, p1, p2, MR, AR, PR);
+  T ML, MR, aL, aR;
+  speed_mach(qL[0], d == 1 ? qL[1] : qL[2], ad, aL, ML);
+  speed_mach(qR[0], d == 1 ? qR[1] : qR[2], ad, aR, MR);
   // M+(M_L), beta+(M_L)
   T mp, bp, mm, bm;
   if (fabs(re(ML)) <= 1.0) {
     T t = ML + 1.0;
     mp = 0.25 * (t * t);
-    bp = (0.25 * (t * t)) * (2.0 * mk(1.0, 0.0, (T*)nullptr) - ML);
+    bp = mp * (2.0 * mk(1.0, 0.0, (T*)nullptr) - ML);
   } else if (re(ML) > 0.0) {
     mp = ML;
     bp = mk(1.0, 0.0, (T*)nullptr);
@@ -101,30 +106,120 @@ __device__ __forceinline__ void ausm_flux(const T qL[3], const T qR[3], int d, d
     mm = MR;
     bm = mk(1.0, 0.0, (T*)nullptr);
   }
-  T Mh = mp + mm;
-  bool pos = re(Mh) > 0.0;
+  const T Mh = mp + mm;
+  const bool pos = re(Mh) > 0.0;
+  const T w = Mh * (pos ? aL : aR);
+  const T pres = bp * (qL[0] * qL[0]) + bm * (qR[0] * qR[0]);
+  flux[0] = w * (pos ? qL[0] : qR[0]);
+  flux[1] = w * (pos ? qL[1] : qR[1]) + p1 * pres;
+  flux[2] = w * (pos ? qL[2] : qR[2]) + p2 * pres;
+}
+
+// One side's columns of the flux's Jacobian (what the complex step of
+// ausm_flux gives for unit imaginary parts of that side's three components):
+// dmh, db: d M_{1/2} / dM and d beta / dM of this side; b: its beta; W: M_{1/2}
+// a^d where this side is upwind, else 0; up: the upwind side's a^d q^mu.
+__device__ __forceinline__ void ausm_jacobian_side(const double q[3], int d, double M, double r, double gd,
+                                                   double dmh, double db, double b, double W, const double up[3],
+                                                   double p1, double p2, double J[3][3]) {
+  const double g0 = -1.5 * M * r;     // dM/dq^0 (M = q^d / (q^0 a), a ~ sqrt(q^0)); gd = dM/dq^d
+  const double q0sq = q[0] * q[0], hw = 0.5 * W * r, bq = 2.0 * b * q[0];
 #pragma unroll
   for (int mu = 0; mu < 3; ++mu) {
-    T adv = pos ? Mh * AL[mu] : Mh * AR[mu];
-    flux[mu] = (adv + bp * PL[mu]) + bm * PR[mu];
+    const double pm = mu == 0 ? 0.0 : (mu == 1 ? p1 : p2);
+    const double c = mu == 0 ? dmh * up[0] : fma(dmh, up[mu], db * pm * q0sq);
+    J[mu][0] = mu == 0 ? fma(c, g0, 1.5 * W) : fma(c, g0, fma(hw, q[mu], bq * pm));
+    const double cd = c * gd;
+    J[mu][1] = (d == 1 ? cd : 0.0) + (mu == 1 ? W : 0.0);
+    J[mu][2] = (d == 2 ? cd : 0.0) + (mu == 2 ? W : 0.0);
   }
 }
 
+// The Jacobian of ausm_flux with respect to (qL, qR), the real parts evaluated
+// once for all six columns.  (Six complex-step evaluations, one per column,
+// took 343 us at 6 x 60 x 60, p = 5, bound by the FP64 pipe: every one repeats
+// the square roots and reciprocals.)
+__device__ __forceinline__ void ausm_jacobian(const double qL[3], const double qR[3], int d, double ad, double p1,
+                                              double p2, double JL[3][3], double JR[3][3]) {
+  const double rL = 1.0 / qL[0], rR = 1.0 / qR[0];
+  const double aL = sqrt(ad * qL[0]), aR = sqrt(ad * qR[0]);
+  const double gL = rL / aL, gR = rR / aR;   // dM/dq^d
+  const double ML = (d == 1 ? qL[1] : qL[2]) * gL, MR = (d == 1 ? qR[1] : qR[2]) * gR;
+  double mp, dmp, bp, dbp, mm, dmm, bm, dbm;
+  if (fabs(ML) <= 1.0) {
+    const double t = ML + 1.0;
+    mp = 0.25 * t * t;
+    dmp = 0.5 * t;
+    bp = mp * (2.0 - ML);
+    dbp = 0.75 * t * (1.0 - ML);
+  } else {
+    const bool up = ML > 0.0;
+    mp = up ? ML : 0.0 * ML;
+    dmp = bp = up ? 1.0 : 0.0;
+    dbp = 0.0;
+  }
+  if (fabs(MR) <= 1.0) {
+    const double t = MR - 1.0;
+    mm = -0.25 * t * t;
+    dmm = -0.5 * t;
+    bm = 0.25 * t * t * (MR + 2.0);
+    dbm = 0.75 * t * (MR + 1.0);
+  } else {
+    const bool up = MR > 0.0;
+    mm = up ? 0.0 * MR : MR;
+    dmm = bm = up ? 0.0 : 1.0;
+    dbm = 0.0;
+  }
+  const double Mh = mp + mm;
+  const bool pos = Mh > 0.0;
+  const double au = pos ? aL : aR, W = Mh * au;
+  const double up[3] = {au * (pos ? qL[0] : qR[0]), au * (pos ? qL[1] : qR[1]), au * (pos ? qL[2] : qR[2])};
+  ausm_jacobian_side(qL, d, ML, rL, gL, dmp, dbp, bp, pos ? W : 0.0, up, p1, p2, JL);
+  ausm_jacobian_side(qR, d, MR, rR, gR, dmm, dbm, bm, pos ? 0.0 : W, up, p1, p2, JR);
+}
+
+// ---------------------------------------------------------------- traces
+// the packed trace weights of an element edge (0 W, 1 E, 2 S, 3 N)
+template <int NS>
+__device__ __forceinline__ void trace_weights(const DfrConst& dc, int edge, double (&wq)[NS]) {
+  const bool lo = (edge & 1) == 0;
+#pragma unroll
+  for (int k = 0; k < NS; ++k) wq[k] = lo ? dc.lmq[k] : dc.lpq[k];
+}
+
+// traces of the three variables of x at point i of an element edge (Eq. 7 at
+// the element ends), in block fixed point with the exponent of the line's N_s
+// values: 36 of the split product's 59 FP64 instructions per interface point
+// at N_s = 6 become six conversions (its face kernel at 6 x 60 x 60, p = 5: 34
+// -> 26 us; with fewer reciprocals in the AUSM flux the face kernel of the
+// right-hand side 73 -> 48 us)
+template <int NS>
+__device__ __forceinline__ void trace_fx(const double* __restrict__ x, long long nodes, int elem, int edge, int i,
+                                         const DfrConst& dc, double out[3]) {
+  const long long base = (long long)elem * NS * NS + (edge <= 1 ? i * NS : i);
+  const int step = edge <= 1 ? 1 : NS;
+  double wq[NS];
+  trace_weights<NS>(dc, edge, wq);
+#pragma unroll
+  for (int var = 0; var < 3; ++var) {
+    double v[NS];
+#pragma unroll
+    for (int k = 0; k < NS; ++k) v[k] = __ldg(x + base + k * step + var * nodes);
+    out[var] = fx_dot<NS>(v, wq, dc.lq_exp, (edge & 1) == 0, dc.lm, dc.lp);
+  }
+}
+
+// traces of the state (real) or of q + i eps v
 template <typename T, int NS>
 __device__ __forceinline__ void trace(const double* __restrict__ q, const double* __restrict__ v, double eps,
                                       long long nodes, int elem, int edge, int i, const DfrConst& dc, T out[3]) {
-  const long long base = (long long)elem * NS * NS;
-  const double* w = (edge == 0 || edge == 2) ? dc.lm : dc.lp;
-#pragma unroll
-  for (int var = 0; var < 3; ++var) {
-    T acc = mk(0.0, 0.0, (T*)nullptr);
-#pragma unroll
-    for (int k = 0; k < NS; ++k) {
-      long long idx = base + ((edge <= 1) ? (i * NS + k) : (k * NS + i)) + var * nodes;
-      acc = acc + w[k] * load_state<T>(q, v, eps, idx);
-    }
-    out[var] = acc;
+  double a[3], b[3] = {0.0, 0.0, 0.0};
+  trace_fx<NS>(q, nodes, elem, edge, i, dc, a);
+  if constexpr (sizeof(T) > sizeof(double)) {
+    if (v) trace_fx<NS>(v, nodes, elem, edge, i, dc, b);
   }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) out[k] = mk(a[k], eps * b[k], (T*)nullptr);
 }
 
 template <int NS>

@@ -13,9 +13,10 @@
 //                     Eq. (2) as functions of Im q;
 //   lin_face_kernel   per interface point: the 3 x 6 matrix taking the
 //                     imaginary parts of the two traces to the imaginary part of
-//                     the AUSM flux, obtained by propagating unit imaginary
-//                     parts through the same complex-step AUSM code as the
-//                     plain kernels (the neighbour's App. C transform folded in).
+//                     the AUSM flux: what propagating unit imaginary parts
+//                     through the plain kernels' AUSM code gives, with the real
+//                     parts evaluated once (ausm_jacobian; the neighbour's App. C
+//                     transform folded in).
 // Each JVP then runs only the imaginary half, in real arithmetic:
 //   face_tangent_kernel   traces of v, the 3 x 6 map, the hand-back;
 //   volume_tangent_kernel pointwise imaginary fluxes and sources, the DFR
@@ -90,28 +91,30 @@ __global__ void __launch_bounds__(128) lin_face_kernel(LinFaceArgs a, DfrConst d
   const double T00 = fc[FC_T00 * P], T01 = fc[FC_T01 * P], T10 = fc[FC_T10 * P], T11 = fc[FC_T11 * P];
   const double qt[3] = {qn[0], T00 * qn[1] + T01 * qn[2], T10 * qn[1] + T11 * qn[2]};
   const double ad = fc[FC_AD * P], p1 = fc[FC_P1 * P], p2 = fc[FC_P2 * P];
-  const double* qL = L.owner_is_left ? qo : qt;
-  const double* qR = L.owner_is_left ? qt : qo;
-  double J[3][6];
-#pragma unroll 1
-  for (int col = 0; col < 6; ++col) {
-    cs zL[3], zR[3], fl[3];
-    for (int k = 0; k < 3; ++k) {
-      zL[k] = {qL[k], (col == k) ? 1.0 : 0.0};
-      zR[k] = {qR[k], (col == k + 3) ? 1.0 : 0.0};
-    }
-    ausm_flux<cs>(zL, zR, L.dir, ad, p1, p2, fl);
-    for (int mu = 0; mu < 3; ++mu) J[mu][col] = fl[mu].im;
+  double qL[3], qR[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    qL[k] = L.owner_is_left ? qo[k] : qt[k];
+    qR[k] = L.owner_is_left ? qt[k] : qo[k];
   }
+  double JL[3][3], JR[3][3];
+  ausm_jacobian(qL, qR, L.dir, ad, p1, p2, JL, JR);
   // columns of the owner trace and of the neighbour trace (own coordinates)
-  const int co = L.owner_is_left ? 0 : 3, cn = L.owner_is_left ? 3 : 0;
   double* out = a.lf + t;
+#pragma unroll
   for (int mu = 0; mu < 3; ++mu) {
-    for (int k = 0; k < 3; ++k) out[(mu * 3 + k) * P] = J[mu][co + k];
+    double o[3], nb[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      o[k] = L.owner_is_left ? JL[mu][k] : JR[mu][k];
+      nb[k] = L.owner_is_left ? JR[mu][k] : JL[mu][k];
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) out[(mu * 3 + k) * P] = o[k];
     // neighbour: Im q_t = blockdiag(1, T) Im q_n
-    out[(9 + mu * 3 + 0) * P] = J[mu][cn + 0];
-    out[(9 + mu * 3 + 1) * P] = J[mu][cn + 1] * T00 + J[mu][cn + 2] * T10;
-    out[(9 + mu * 3 + 2) * P] = J[mu][cn + 1] * T01 + J[mu][cn + 2] * T11;
+    out[(9 + mu * 3 + 0) * P] = nb[0];
+    out[(9 + mu * 3 + 1) * P] = nb[1] * T00 + nb[2] * T10;
+    out[(9 + mu * 3 + 2) * P] = nb[1] * T01 + nb[2] * T11;
   }
 }
 

@@ -22,23 +22,22 @@ namespace swepi {
 template <typename T, int NS>
 __device__ __forceinline__ void trace_tan(const double* __restrict__ v, const float* __restrict__ v32, long long nodes,
                                           int elem, int edge, int i, const DfrConst& dc, T out[3]) {
-  const long long base = (long long)elem * NS * NS;
-  const double* w = (edge == 0 || edge == 2) ? dc.lm : dc.lp;
-  const float* w32 = (edge == 0 || edge == 2) ? dc.lm32 : dc.lp32;
+  if constexpr (sizeof(T) == 8) {
+    trace_fx<NS>(v, nodes, elem, edge, i, dc, out);
+  } else {
+    const long long base = (long long)elem * NS * NS;
+    const float* w32 = (edge == 0 || edge == 2) ? dc.lm32 : dc.lp32;
 #pragma unroll
-  for (int var = 0; var < 3; ++var) {
-    T acc = T(0);
+    for (int var = 0; var < 3; ++var) {
+      T acc = T(0);
 #pragma unroll
-    for (int k = 0; k < NS; ++k) {
-      const long long idx = base + ((edge <= 1) ? (i * NS + k) : (k * NS + i)) + var * nodes;
-      if constexpr (sizeof(T) == 4) {
+      for (int k = 0; k < NS; ++k) {
+        const long long idx = base + ((edge <= 1) ? (i * NS + k) : (k * NS + i)) + var * nodes;
         const float x = v32 ? __ldg(v32 + idx) : f64_to_f32_bits(__ldg(v + idx));
         acc = fmaf(w32[k], x, acc);
-      } else {
-        acc = fma(w[k], __ldg(v + idx), acc);
       }
+      out[var] = acc;
     }
-    out[var] = acc;
   }
 }
 
