@@ -71,17 +71,22 @@ __global__ void __launch_bounds__(128) face_flux_kernel(FaceArgs a, DfrConst dc)
     ausm_flux<T>(qo, qt, L.dir, ad, p1, p2, fl);
   else
     ausm_flux<T>(qt, qo, L.dir, ad, p1, p2, fl);
-  const double sig = fc[FC_SIG * P];
-  const double M00 = fc[FC_M00 * P], M01 = fc[FC_M01 * P], M10 = fc[FC_M10 * P], M11 = fc[FC_M11 * P];
   double f0 = part(fl[0]), f1 = part(fl[1]), f2 = part(fl[2]);
   double* fo = a.fb + ((long long)L.owner * 4 + L.owner_edge) * 3 * NS + i;
   fo[0] = f0;
   fo[NS] = f1;
   fo[2 * NS] = f2;
+  if (L.handback) {   // across panels: the neighbour's components (App. C); within a panel the same flux
+    const double M00 = fc[FC_M00 * P], M01 = fc[FC_M01 * P], M10 = fc[FC_M10 * P], M11 = fc[FC_M11 * P];
+    const double g1 = M00 * f1 + M01 * f2, g2 = M10 * f1 + M11 * f2;
+    f0 *= fc[FC_SIG * P];
+    f1 = g1;
+    f2 = g2;
+  }
   double* fn = a.fb + ((long long)L.nbr * 4 + L.nbr_edge) * 3 * NS + in;
-  fn[0] = sig * f0;
-  fn[NS] = M00 * f1 + M01 * f2;
-  fn[2 * NS] = M10 * f1 + M11 * f2;
+  fn[0] = f0;
+  fn[NS] = f1;
+  fn[2 * NS] = f2;
 }
 
 // ---------------------------------------------------------------- volume

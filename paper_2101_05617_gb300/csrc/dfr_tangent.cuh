@@ -78,29 +78,37 @@ __device__ __forceinline__ void face_tangent_body(const TanFaceArgs<T>& a, const
     s = fma(lf[(9 + mu * 3 + 2) * P], vn[2], s);
     f[mu] = s;
   }
-  T sig, M00, M01, M10, M11;
-  if constexpr (sizeof(T) == 4) {   // FP32 copies of the hand-back coefficients after the 18 map rows
-    M00 = lf[18 * P];
-    M01 = lf[19 * P];
-    M10 = lf[20 * P];
-    M11 = lf[21 * P];
-    sig = lf[22 * P];
-  } else {
-    const double* fc = a.fc + t;
-    sig = fc[FC_SIG * P];
-    M00 = fc[FC_M00 * P];
-    M01 = fc[FC_M01 * P];
-    M10 = fc[FC_M10 * P];
-    M11 = fc[FC_M11 * P];
-  }
   T* fo = a.fb + ((long long)L.owner * 4 + L.owner_edge) * 3 * NS + i;
   fo[0] = f[0];
   fo[NS] = f[1];
   fo[2 * NS] = f[2];
+  // across panels the neighbour's components (App. C); within a panel the
+  // transform is the identity and its five coefficients are not read
+  if (L.handback) {
+    T sig, M00, M01, M10, M11;
+    if constexpr (sizeof(T) == 4) {   // FP32 copies of the hand-back coefficients after the 18 map rows
+      M00 = lf[18 * P];
+      M01 = lf[19 * P];
+      M10 = lf[20 * P];
+      M11 = lf[21 * P];
+      sig = lf[22 * P];
+    } else {
+      const double* fc = a.fc + t;
+      sig = fc[FC_SIG * P];
+      M00 = fc[FC_M00 * P];
+      M01 = fc[FC_M01 * P];
+      M10 = fc[FC_M10 * P];
+      M11 = fc[FC_M11 * P];
+    }
+    const T g1 = M00 * f[1] + M01 * f[2], g2 = M10 * f[1] + M11 * f[2];
+    f[0] = sig * f[0];
+    f[1] = g1;
+    f[2] = g2;
+  }
   T* fn = a.fb + ((long long)L.nbr * 4 + L.nbr_edge) * 3 * NS + in;
-  fn[0] = sig * f[0];
-  fn[NS] = M00 * f[1] + M01 * f[2];
-  fn[2 * NS] = M10 * f[1] + M11 * f[2];
+  fn[0] = f[0];
+  fn[NS] = f[1];
+  fn[2 * NS] = f[2];
 }
 
 template <typename T>

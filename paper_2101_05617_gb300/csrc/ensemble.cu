@@ -315,10 +315,13 @@ __device__ void scale_task(const EnsDesc& d, EnsDyn& y, unsigned int local, EnsC
   const bool skip = __ldcg(d.flags) != 0;
   const long long N = d.n + d.p;
   double acc = 0.0;
+  __shared__ double s_r;   // one division per task (a chain of FP64 instructions)
+  if (threadIdx.x == 0) s_r = skip ? 0.0 : 1.0 / __ldcg(d.H + (long long)(j + 1) * d.ldh + j);
+  __syncthreads();
   if (!skip) {
     double* z = d.V + (long long)(j + 1) * d.ldv;
     const double* VB = d.V + (long long)j * d.ldv;
-    const double r = 1.0 / __ldcg(d.H + (long long)(j + 1) * d.ldh + j);
+    const double r = s_r;
     const long long i0 = (long long)local * d.vec_len, i1 = min(i0 + d.vec_len, N);
     acc = scale_dot_range(z, VB, r, i0 + threadIdx.x, i1, BLOCK);
   }

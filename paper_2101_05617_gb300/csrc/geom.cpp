@@ -354,7 +354,7 @@ int build_tables(Ctx& c) {
       edge_element(c, f.ea, e, oe2, oe1);
       edge_element(c, f.eb, f.rev ? ne - 1 - e : e, ne2, ne1);
       FaceLine L{(int)elem_index(c, f.pa, oe2, oe1), f.ea, (int)elem_index(c, f.pb, ne2, ne1), f.eb,
-                 f.rev, da, (f.ea == 1 || f.ea == 3) ? 1 : 0, 0};
+                 f.rev, da, (f.ea == 1 || f.ea == 3) ? 1 : 0, 1};
       double edge_c = (f.ea == 1 || f.ea == 3) ? kQuarterPi : -kQuarterPi;
       for (int i = 0; i < ns; ++i) {
         double t = line_coord(c, e, i);

@@ -386,16 +386,16 @@ int build(Ctx& c, KGraph& G, int p, int iop, bool fp32, int mmax) {
     if (int r = capture_iter_jvp(c, kd, f, fp32, w3, p, s)) return r;
     if (fp32) {   // complex64-bulk form: the dots in a pass of their own
       if (w3)
-        kg_dots_kernel<true><<<RED_BLOCKS, kRedThreads, 0, s>>>(kd, f);
+        kg_dots_kernel<true><<<red_blocks(f.N), kRedThreads, 0, s>>>(kd, f);
       else
-        kg_dots_kernel<false><<<RED_BLOCKS, kRedThreads, 0, s>>>(kd, f);
+        kg_dots_kernel<false><<<red_blocks(f.N), kRedThreads, 0, s>>>(kd, f);
     }
     if (w3) {
-      kg_update_kernel<true><<<RED_BLOCKS, kRedThreads, 0, s>>>(kd, f);
-      kg_scale_kernel<true><<<RED_BLOCKS, kRedThreads, 0, s>>>(kd, f);
+      kg_update_kernel<true><<<red_blocks(f.N), kRedThreads, 0, s>>>(kd, f);
+      kg_scale_kernel<true><<<red_blocks(f.N), kRedThreads, 0, s>>>(kd, f);
     } else {
-      kg_update_kernel<false><<<RED_BLOCKS, kRedThreads, 0, s>>>(kd, f);
-      kg_scale_kernel<false><<<RED_BLOCKS, kRedThreads, 0, s>>>(kd, f);
+      kg_update_kernel<false><<<red_blocks(f.N), kRedThreads, 0, s>>>(kd, f);
+      kg_scale_kernel<false><<<red_blocks(f.N), kRedThreads, 0, s>>>(kd, f);
     }
     kg_advance_kernel<<<1, 1, 0, s>>>(kd, f, hi);
     return cuda_status(cudaGetLastError());

@@ -250,7 +250,7 @@ double fp64_fma_peak_tflops() {
 
 int launch_dot(Ctx& c, const double* x, const double* y, long long n, double* dst, const int* skip, cudaStream_t s) {
   RedOut o{dst, 0.0, nullptr, 0};
-  reduce_kernel<OP_DOT><<<RED_BLOCKS, RED_THREADS, 0, s>>>(x, y, n, c.d_partials, (unsigned int*)(c.d_flags + 8), o,
+  reduce_kernel<OP_DOT><<<red_blocks(n), RED_THREADS, 0, s>>>(x, y, n, c.d_partials, (unsigned int*)(c.d_flags + 8), o,
                                                           skip);
   c.launches++;
   return cuda_status(cudaGetLastError());
@@ -259,7 +259,7 @@ int launch_dot(Ctx& c, const double* x, const double* y, long long n, double* ds
 int launch_norm2(Ctx& c, const double* x, long long n, double* dst, double tol, int* happy, int happy_value,
                  const int* skip, cudaStream_t s) {
   RedOut o{dst, tol, happy, happy_value};
-  reduce_kernel<OP_NORM2><<<RED_BLOCKS, RED_THREADS, 0, s>>>(x, nullptr, n, c.d_partials,
+  reduce_kernel<OP_NORM2><<<red_blocks(n), RED_THREADS, 0, s>>>(x, nullptr, n, c.d_partials,
                                                             (unsigned int*)(c.d_flags + 8), o, skip);
   c.launches++;
   return cuda_status(cudaGetLastError());
@@ -267,7 +267,7 @@ int launch_norm2(Ctx& c, const double* x, long long n, double* dst, double tol, 
 
 int launch_norm1(Ctx& c, const double* x, long long n, double* dst, cudaStream_t s) {
   RedOut o{dst, 0.0, nullptr, 0};
-  reduce_kernel<OP_NORM1><<<RED_BLOCKS, RED_THREADS, 0, s>>>(x, nullptr, n, c.d_partials,
+  reduce_kernel<OP_NORM1><<<red_blocks(n), RED_THREADS, 0, s>>>(x, nullptr, n, c.d_partials,
                                                             (unsigned int*)(c.d_flags + 8), o, nullptr);
   c.launches++;
   return cuda_status(cudaGetLastError());
@@ -296,7 +296,7 @@ int launch_update_norm(Ctx& c, double* z, const double* VA, const double* VB, co
     e1 = prof_event(c);
     cudaEventRecord(e0, s);
   }
-  if (launch_pdl(update_norm_kernel, dim3(RED_BLOCKS), dim3(RED_THREADS), s, z, VA, VB, h1, h2, N, c.d_partials,
+  if (launch_pdl(update_norm_kernel, dim3(red_blocks(N)), dim3(RED_THREADS), s, z, VA, VB, h1, h2, N, c.d_partials,
                  (unsigned int*)(c.d_flags + 8), hsub, tol, c.d_flags, happy_value, VC, h0) != cudaSuccess)
     return SW_ECUDA;
   if (prof_on(c, PK_ORTH)) {
@@ -315,7 +315,7 @@ int launch_scale_dot(Ctx& c, double* z, const double* VB, const double* hsub, lo
     e1 = prof_event(c);
     cudaEventRecord(e0, s);
   }
-  if (launch_pdl(scale_dot_kernel, dim3(RED_BLOCKS), dim3(RED_THREADS), s, z, VB, hsub, N, c.d_partials,
+  if (launch_pdl(scale_dot_kernel, dim3(red_blocks(N)), dim3(RED_THREADS), s, z, VB, hsub, N, c.d_partials,
                  (unsigned int*)(c.d_flags + 8), c_out, c.d_flags, VA, c2_out, z32) != cudaSuccess)
     return SW_ECUDA;
   if (prof_on(c, PK_ORTH)) {
@@ -350,7 +350,7 @@ int launch_orth_dots(Ctx& c, const double* z, const double* VB, const double* VA
     e1 = prof_event(c);
     cudaEventRecord(e0, s);
   }
-  if (launch_pdl(orth_dots_kernel, dim3(RED_BLOCKS), dim3(RED_THREADS), s, z, VB, VA, VC, N, c.d_partials,
+  if (launch_pdl(orth_dots_kernel, dim3(red_blocks(N)), dim3(RED_THREADS), s, z, VB, VA, VC, N, c.d_partials,
                  reinterpret_cast<unsigned int*>(c.d_flags + 8), static_cast<const int*>(c.d_flags), h0_out, h1_out,
                  h2_out, cdot_out, cdot2_out, cprevAC) != cudaSuccess)
     return SW_ECUDA;
@@ -372,7 +372,7 @@ int launch_orth3_fused(Ctx& c, double* z, const double* VA, const double* VB, co
     cudaEventRecord(e0, s);
   }
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(RED_BLOCKS);
+  cfg.gridDim = dim3(red_blocks(N));
   cfg.blockDim = dim3(RED_THREADS);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
@@ -404,7 +404,7 @@ int launch_orth_fused(Ctx& c, double* z, const double* VA, const double* VB, con
     cudaEventRecord(e0, s);
   }
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(RED_BLOCKS);
+  cfg.gridDim = dim3(red_blocks(N));
   cfg.blockDim = dim3(RED_THREADS);
   cfg.stream = s;
   cudaLaunchAttribute at[1];

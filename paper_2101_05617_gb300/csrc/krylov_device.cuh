@@ -77,7 +77,10 @@ __device__ __forceinline__ void block_sums_k(double v[K]) {
 // indices i0, i0 + stride, ... < i1 of one thread, eight elements in flight
 // with two window vectors, four with three (the 64-register budget of the
 // cooperative grid); the order of the operations is the same either way
-// (z was written by another kernel or CTA: read through L2).
+// (z was written by another kernel or CTA: read through L2).  What is left
+// after the full batches goes as one guarded batch: a thread has 15 entries at
+// 6 x 60 x 60, p = 5 and four at 6 x 30 x 30, so a one-by-one remainder made
+// most of them wait for memory one after another.
 //   z -= h0 VC + h1 VA + h2 VB (VC, VA may be null; oldest first); returns the
 //   thread's sum of z_i^2
 // HA, HC: VA, VC present (compiled in, so that no guarded-off FP64
@@ -87,7 +90,7 @@ __device__ __forceinline__ double mgs_update_range_t(double* __restrict__ z, con
                                                      const double* __restrict__ VB, double h1, double h2, long long i,
                                                      long long i1, long long stride, const double* __restrict__ VC,
                                                      double h0) {
-  constexpr int D = HC ? 4 : 8;   // entries in flight per thread
+    constexpr int D = HC ? 4 : 8;   // entries in flight per thread
   double acc = 0.0;
   for (; i + (D - 1) * stride < i1; i += D * stride) {
     double v[D], b[D], a[D], c[D];
@@ -107,13 +110,27 @@ __device__ __forceinline__ double mgs_update_range_t(double* __restrict__ z, con
       acc = fma(v[k], v[k], acc);
     }
   }
-  for (; i < i1; i += stride) {
-    double v = __ldcg(z + i);
-    if (HC) v = fma(-h0, VC[i], v);
-    if (HA) v = fma(-h1, VA[i], v);
-    v = fma(-h2, VB[i], v);
-    z[i] = v;
-    acc = fma(v, v, acc);
+  if (i < i1) {
+    double v[D - 1], b[D - 1], a[D - 1], c[D - 1];
+#pragma unroll
+    for (int k = 0; k < D - 1; ++k) {
+      const long long j = i + k * stride;
+      if (j >= i1) break;
+      v[k] = __ldcg(z + j);
+      b[k] = VB[j];
+      if (HA) a[k] = VA[j];
+      if (HC) c[k] = VC[j];
+    }
+#pragma unroll
+    for (int k = 0; k < D - 1; ++k) {
+      const long long j = i + k * stride;
+      if (j >= i1) break;
+      if (HC) v[k] = fma(-h0, c[k], v[k]);
+      if (HA) v[k] = fma(-h1, a[k], v[k]);
+      v[k] = fma(-h2, b[k], v[k]);
+      z[j] = v[k];
+      acc = fma(v[k], v[k], acc);
+    }
   }
   return acc;
 }
@@ -156,12 +173,26 @@ __device__ __forceinline__ double scale_dot_range(double* __restrict__ z, const 
         acc2 = fma(v[k], a[k], acc2);
       }
     }
-    for (; i < i1; i += stride) {
-      const double v = __ldcg(z + i) * r;
-      z[i] = v;
-      if (z32) z32[i] = f64_to_f32_bits(v);
-      acc = fma(v, VB[i], acc);
-      acc2 = fma(v, VA[i], acc2);
+    if (i < i1) {
+      double v[3], b[3], a[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const long long j = i + k * stride;
+        if (j >= i1) break;
+        v[k] = __ldcg(z + j);
+        b[k] = VB[j];
+        a[k] = VA[j];
+      }
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const long long j = i + k * stride;
+        if (j >= i1) break;
+        v[k] *= r;
+        z[j] = v[k];
+        if (z32) z32[j] = f64_to_f32_bits(v[k]);
+        acc = fma(v[k], b[k], acc);
+        acc2 = fma(v[k], a[k], acc2);
+      }
     }
     *za = acc2;
     return acc;
@@ -182,11 +213,24 @@ __device__ __forceinline__ double scale_dot_range(double* __restrict__ z, const 
       acc = fma(v[k], b[k], acc);
     }
   }
-  for (; i < i1; i += stride) {
-    const double v = __ldcg(z + i) * r;
-    z[i] = v;
-    if (z32) z32[i] = f64_to_f32_bits(v);
-    acc = fma(v, VB[i], acc);
+  if (i < i1) {
+    double v[3], b[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const long long j = i + k * stride;
+      if (j >= i1) break;
+      v[k] = __ldcg(z + j);
+      b[k] = VB[j];
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const long long j = i + k * stride;
+      if (j >= i1) break;
+      v[k] *= r;
+      z[j] = v[k];
+      if (z32) z32[j] = f64_to_f32_bits(v[k]);
+      acc = fma(v[k], b[k], acc);
+    }
   }
   return acc;
 }
@@ -243,13 +287,31 @@ __device__ __forceinline__ void scale_dot_dev(double* __restrict__ z, const doub
                                               double* c2_out, float* __restrict__ z32) {
   // through L2: in the fused launch another CTA has just written them
   if (__ldcg(happy)) return;
-  const double r = 1.0 / __ldcg(hsub);
+  // one division per CTA: a reciprocal is a chain of FP64 instructions, and in
+  // every warp it held the pipe as long as the pass's own work on small grids
+  __shared__ double s_r;
+  if (threadIdx.x == 0) s_r = 1.0 / __ldcg(hsub);
+  __syncthreads();
+  const double r = s_r;
   if (!c_out) {   // scale only (the next volume kernel forms the dots)
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-      const double v = __ldcg(z + i) * r;
-      z[i] = v;
-      if (z32) z32[i] = f64_to_f32_bits(v);
+    constexpr int D = 8;   // entries in flight per thread, the last batch guarded
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += D * stride) {
+      double v[D];
+#pragma unroll
+      for (int k = 0; k < D; ++k) {
+        const long long j = i + k * stride;
+        if (j < n) v[k] = __ldcg(z + j);
+      }
+#pragma unroll
+      for (int k = 0; k < D; ++k) {
+        const long long j = i + k * stride;
+        if (j < n) {
+          v[k] *= r;
+          z[j] = v[k];
+          if (z32) z32[j] = f64_to_f32_bits(v[k]);
+        }
+      }
     }
     return;
   }
@@ -363,18 +425,29 @@ __device__ __forceinline__ void orth_dots_range_t(const double* __restrict__ z, 
       }
     }
   }
-  for (; i < i1; i += stride) {
-    const double zz = __ldcg(z + i), b = VB[i];
-    db = fma(zz, b, db);
-    if (HA) {
-      const double a = VA[i];
-      da = fma(zz, a, da);
-      dab = fma(b, a, dab);
+  if (i < i1) {
+    double zz[3], b[3], a[3], c[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const long long j = i + k * stride;
+      if (j >= i1) break;
+      zz[k] = __ldcg(z + j);
+      b[k] = VB[j];
+      if (HA) a[k] = VA[j];
+      if (HC) c[k] = VC[j];
     }
-    if (HC) {
-      const double c = VC[i];
-      dc = fma(zz, c, dc);
-      dbc = fma(b, c, dbc);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      if (i + k * stride >= i1) break;
+      db = fma(zz[k], b[k], db);
+      if (HA) {
+        da = fma(zz[k], a[k], da);
+        dab = fma(b[k], a[k], dab);
+      }
+      if (HC) {
+        dc = fma(zz[k], c[k], dc);
+        dbc = fma(b[k], c[k], dbc);
+      }
     }
   }
   s[0] = da;

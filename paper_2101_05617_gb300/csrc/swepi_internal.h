@@ -65,7 +65,7 @@ struct FaceLine {
   int reversed;            // neighbour point index = N_s-1-i
   int dir;                 // owner normal direction (1 or 2)
   int owner_is_left;       // owner edge is E or N
-  int pad;
+  int handback;            // 1: panels differ, the flux handed to the neighbour is transformed (0: the same flux)
 };
 
 // Small DFR constants passed by value to the kernels.
@@ -288,6 +288,14 @@ int launch_jvp_fb(Ctx& c, const double* q, const double* v, double eps, double* 
 
 // ---- Krylov kernels (krylov.cu)
 constexpr int RED_BLOCKS = 608;   // 4 x 152 SMs
+// CTAs of a reduction or vector pass over n entries (256 threads each): two
+// entries a thread until the GPU is full.  Every CTA takes a ticket, and in the
+// cooperative pass waits for the last one, so idle CTAs cost time: at n = 4608
+// (6 x 4 x 4, p = 3) the two passes take 14.4 us with ten CTAs, 18.4 with 608.
+inline int red_blocks(long long n) {
+  const long long b = (n + 511) / 512;
+  return (int)(b < 1 ? 1 : (b > RED_BLOCKS ? RED_BLOCKS : b));
+}
 int launch_dot(Ctx& c, const double* x, const double* y, long long n, double* dst, const int* skip,
                cudaStream_t s);
 int launch_norm2(Ctx& c, const double* x, long long n, double* dst, double tol, int* happy,
