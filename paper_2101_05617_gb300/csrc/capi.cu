@@ -311,6 +311,7 @@ void sw_free(sw_ctx_t c) {
   if (c->d_lin_node32) cudaFree(c->d_lin_node32);
   if (c->d_lin_face32) cudaFree(c->d_lin_face32);
   if (c->d_b32) cudaFree(c->d_b32);
+  if (c->d_v32) cudaFree(c->d_v32);
   if (c->d_V32) cudaFree(c->d_V32);
   for (double* p : ptrs)
     if (p) cudaFree(p);
@@ -787,6 +788,14 @@ int sw_jvp_linearized(sw_ctx_t c, const double* v, double* Jv, void* stream) {
   if (!c->linearized) return SW_EINVAL;
   if (int rc = check_device(*c)) return rc;
   AugEpilogue ep;
+  if (c->jvp_mode == 2) {
+    // the FP32 kernels read each entry of v several times: one FP32 copy (the
+    // rounding they would do themselves, so the same result bit for bit)
+    // instead of a conversion at every use.  6 x 60 x 60, p = 5: the product 54
+    // -> 36 us (its face kernel 29 -> 12 us)
+    if (int rc = launch_to_float(*c, v, c->d_v32, c->n, as_stream(stream))) return rc;
+    ep.v32 = c->d_v32;
+  }
   return launch_jvp_lin(*c, v, Jv, ep, as_stream(stream), c->jvp_mode == 2);
 }
 

@@ -360,6 +360,7 @@ int launch_linearize(Ctx& c, const double* q, cudaStream_t s) {
       return SW_ENOMEM;
     if (!c.d_lin_face32 && cudaMalloc(&c.d_lin_face32, sizeof(float) * 23 * c.nfacepts) != cudaSuccess)
       return SW_ENOMEM;
+    if (!c.d_v32 && cudaMalloc(&c.d_v32, sizeof(float) * c.n) != cudaSuccess) return SW_ENOMEM;
     to_float_kernel<<<1024, 256, 0, s>>>(c.d_lin_node, c.d_lin_node32, (long long)LN_COUNT * c.nodes);
     to_float_kernel<<<1024, 256, 0, s>>>(c.d_lin_face, c.d_lin_face32, 18LL * c.nfacepts);
     // M00, M01, M10, M11, sigma (consecutive rows of the face table) after the map rows

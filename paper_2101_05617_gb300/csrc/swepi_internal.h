@@ -141,6 +141,7 @@ struct Ctx {
   float* d_lin_face32 = nullptr;    // [23][nfacepts]: the 18 flux-map rows, then M00, M01, M10, M11, sigma
   float* d_V32 = nullptr;           // FP32 copy of the Krylov basis [vcap][ldv] (complex64-bulk form)
   int v32_cap = 0;                  // rows allocated in d_V32
+  float* d_v32 = nullptr;           // FP32 copy of the vector of a single complex64-bulk product [n]
   float* d_b32 = nullptr;           // FP32 copies of nu * b_l of the current phi-function call [MAX_NB][n]
   int b32_cap = 0;                  // vectors allocated in d_b32
   // device-driven phi-function solver (kiops_graph.cu)
