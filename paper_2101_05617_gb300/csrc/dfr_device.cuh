@@ -229,7 +229,7 @@ struct VolShape {
 };
 
 
-template <int THREADS, bool W3, bool CD>
+template <int THREADS, bool W3>
 __device__ __forceinline__ void epilogue_finish(const AugEpilogue& ep, double da, double db, double dcc,
                                                 unsigned int blk, unsigned int nblk, double dab, double dbc,
                                                 double* sbuf);
@@ -243,9 +243,7 @@ __device__ __forceinline__ void epilogue_finish(const AugEpilogue& ep, double da
 // SCALED: the caller has already multiplied res by scale.  W3: compiled for
 // the window of three (dotC may be set); W3 = false drops that code.  B64:
 // the b-column terms are added here in FP64; false: the caller has added them
-// already (the FP32 kernels of the complex64-bulk form, from ep.b32).  CD:
-// compiled to form the V . V products when ep.cdot_out asks for them (the
-// complex64-bulk kernels); without it the block sums carry three values.
+// already (the FP32 kernels of the complex64-bulk form, from ep.b32).
 // the tail coefficients nu * y_l of the augmented operator into coef[MAX_NB]
 // (shared memory; the caller synchronises before reading them)
 __device__ __forceinline__ void epilogue_coefs(const AugEpilogue& ep, double* coef) {
@@ -257,9 +255,12 @@ __device__ __forceinline__ void epilogue_coefs(const AugEpilogue& ep, double* co
 
 // Per-node half of the volume epilogue: o = res + sum_l coef_l b_l (B64),
 // stored at out, and this node's terms of the window dots added to the
-// thread's partial sums (da = z . V_{j-1}, db = z . V_j, dcc = z . V_{j-2},
-// and with CD the V . V products dab, dbc).
-template <bool W3, bool B64, bool CD>
+// thread's partial sums (da = z . V_{j-1}, db = z . V_j, dcc = z . V_{j-2} and
+// the window's own products dab = V_j . V_{j-1}, dbc = V_j . V_{j-2}).  The
+// window's products are formed here, where its vectors are read anyway: as sums
+// of the scale pass they cost that pass a second read of V_j and a second
+// grid-wide reduction on the critical path (6 x 30 x 30: 3 us of 21).
+template <bool W3, bool B64>
 __device__ __forceinline__ void epilogue_node(const AugEpilogue& ep, const double* coef, long long idx, long long N,
                                               const double res[3], double* __restrict__ out, double& da, double& db,
                                               double& dcc, double& dab, double& dbc) {
@@ -277,7 +278,6 @@ __device__ __forceinline__ void epilogue_node(const AugEpilogue& ep, const doubl
       for (int mu = 0; mu < 3; ++mu) ob[mu] = fma(cl, bl[idx + mu * N], ob[mu]);
     }
   }
-  const bool cd = CD && ep.cdot_out != nullptr;
 #pragma unroll
   for (int mu = 0; mu < 3; ++mu) {
     const double o = ob[mu];
@@ -288,18 +288,18 @@ __device__ __forceinline__ void epilogue_node(const AugEpilogue& ep, const doubl
       if (ep.dotA) {
         const double va = ep.dotA[idx + mu * N];
         da = fma(o, va, da);
-        if (cd) dab = fma(vb, va, dab);
+        dab = fma(vb, va, dab);
       }
       if (W3 && ep.dotC) {
         const double vc = ep.dotC[idx + mu * N];
         dcc = fma(o, vc, dcc);
-        if (cd) dbc = fma(vb, vc, dbc);
+        dbc = fma(vb, vc, dbc);
       }
     }
   }
 }
 
-template <int THREADS, bool SCALED = false, bool W3 = false, bool B64 = true, bool CD = false>
+template <int THREADS, bool SCALED = false, bool W3 = false, bool B64 = true>
 __device__ __forceinline__ void volume_epilogue(const AugEpilogue& ep, bool active, long long idx, long long N,
                                                 const double res[3], double* __restrict__ out, unsigned int blk,
                                                 unsigned int nblk) {
@@ -311,10 +311,10 @@ __device__ __forceinline__ void volume_epilogue(const AugEpilogue& ep, bool acti
     double r[3];
 #pragma unroll
     for (int mu = 0; mu < 3; ++mu) r[mu] = SCALED ? res[mu] : ep.scale * res[mu];
-    epilogue_node<W3, B64, CD>(ep, coef, idx, N, r, out, da, db, dcc, dab, dbc);
+    epilogue_node<W3, B64>(ep, coef, idx, N, r, out, da, db, dcc, dab, dbc);
   }
-  __shared__ double sred[(CD ? 5 : 3) * THREADS];
-  epilogue_finish<THREADS, W3, CD>(ep, da, db, dcc, blk, nblk, dab, dbc, sred);
+  __shared__ double sred[(W3 ? 5 : 3) * THREADS];
+  epilogue_finish<THREADS, W3>(ep, da, db, dcc, blk, nblk, dab, dbc, sred);
 }
 
 // Sums of K values over the block in a fixed order, through shared scratch of
@@ -347,34 +347,34 @@ __device__ __forceinline__ void block_sums(double v[K], double* sbuf) {
 }
 
 // Second half of the volume epilogue (all threads of the block call it, with
-// their partial window dots da = z . V_{j-1}, db = z . V_j, dcc = z . V_{j-2}
-// over their nodes, and -- when ep.cdot_out is set -- dab = V_j . V_{j-1} and
-// dbc = V_j . V_{j-2}): the shift of the augmented tail, the tail's share of
-// the dots, the block sums and -- in the last block to finish -- the modified
-// Gram-Schmidt coefficients (with the V . V products of this launch when they
-// are formed here, else those stored by the scale pass).  sbuf: K * THREADS
-// doubles of shared scratch, K = 5 with CD, else 3.
-template <int THREADS, bool W3, bool CD>
+// their partial sums over their nodes, see epilogue_node): the shift of the
+// augmented tail, the tail's share of the dots, the block sums and -- in the
+// last block to finish -- the modified Gram-Schmidt coefficients.  sbuf: K *
+// THREADS doubles of shared scratch, K = 5 with W3, else 3.
+template <int THREADS, bool W3>
 __device__ __forceinline__ void epilogue_finish(const AugEpilogue& ep, double da, double db, double dcc,
                                                 unsigned int blk, unsigned int nblk, double dab, double dbc,
                                                 double* sbuf) {
   if (ep.tail_out && blk == 0 && threadIdx.x < ep.p)
     ep.tail_out[threadIdx.x] = (threadIdx.x + 1 < ep.p) ? ep.tail_in[threadIdx.x + 1] : 0.0;
   if (!ep.dotB) return;   // uniform over the grid
-  const bool cd = CD && ep.cdot_out != nullptr;   // uniform over the grid
   if (blk == 0 && threadIdx.x == 0) {
     for (int l = 0; l < ep.p; ++l) {
       const double zt = (l + 1 < ep.p) ? ep.tail_in[l + 1] : 0.0;
       db = fma(zt, ep.dotB[ep.n + l], db);
-      if (ep.dotA) da = fma(zt, ep.dotA[ep.n + l], da);
-      if (W3 && ep.dotC) dcc = fma(zt, ep.dotC[ep.n + l], dcc);
-      if (cd && ep.dotA) dab = fma(ep.tail_in[l], ep.dotA[ep.n + l], dab);
-      if (cd && W3 && ep.dotC) dbc = fma(ep.tail_in[l], ep.dotC[ep.n + l], dbc);
+      if (ep.dotA) {
+        da = fma(zt, ep.dotA[ep.n + l], da);
+        dab = fma(ep.dotB[ep.n + l], ep.dotA[ep.n + l], dab);
+      }
+      if (W3 && ep.dotC) {
+        dcc = fma(zt, ep.dotC[ep.n + l], dcc);
+        dbc = fma(ep.dotB[ep.n + l], ep.dotC[ep.n + l], dbc);
+      }
     }
   }
-  constexpr int K = CD ? 5 : 3;
+  constexpr int K = W3 ? 5 : 3;
   __shared__ bool last;
-  double v[5] = {da, db, dcc, dab, dbc};
+  double v[5] = {da, db, dab, dcc, dbc};
   block_sums<THREADS, K>(v, sbuf);
   if (threadIdx.x == 0) {
 #pragma unroll
@@ -394,27 +394,18 @@ __device__ __forceinline__ void epilogue_finish(const AugEpilogue& ep, double da
   __syncthreads();   // the scratch is reused
   block_sums<THREADS, K>(u, sbuf);
   if (threadIdx.x == 0) {
-    const double a = u[0], b = u[1], c3 = u[2];
-    const bool three = W3 && ep.dotC != nullptr;
-    double cprev = 0.0, cprevC = 0.0;
-    if (ep.dotA) {
-      cprev = cd ? u[3] : *ep.cprev;
-      if (cd) *ep.cdot_out = u[3];   // V_j . V_{j-1}
-    }
-    if (three) {
-      cprevC = cd ? u[4] : *ep.cprevC;
-      if (cd) *ep.cdot2_out = u[4];   // V_j . V_{j-2}
-    }
+    const double a = u[0], b = u[1], vab = u[2];
+    if (ep.dotA) *ep.cdot_out = vab;   // V_j . V_{j-1}: V_{j-1} . V_{j-2} of the next iteration
     // modified Gram-Schmidt coefficients, oldest vector first
-    if (three) {
-      const double h0 = c3;                               // V_{j-2} . z
+    if (W3 && ep.dotC != nullptr) {
+      const double h0 = u[3];                             // V_{j-2} . z
       const double h1 = a - h0 * (*ep.cprevAC);            // V_{j-1} . (z - h0 V_{j-2})
       *ep.h0_out = h0;
       *ep.h1_out = h1;
-      *ep.h2_out = b - h0 * cprevC - h1 * cprev;
+      *ep.h2_out = b - h0 * u[4] - h1 * vab;
     } else if (ep.dotA) {
       *ep.h1_out = a;
-      *ep.h2_out = b - a * cprev;   // V_j . (z - h1 V_{j-1})
+      *ep.h2_out = b - a * vab;   // V_j . (z - h1 V_{j-1})
     } else {
       *ep.h2_out = b;
     }

@@ -413,7 +413,7 @@ __device__ __forceinline__ void volume_tangent_body(const TanVolArgs<T>& a, cons
     fx_sweep<NS>(sm.sF[le], &sm.sB[le][0][0][0], k1, k2, sm.sD[k1], sm.sD[k2], dc, dscale, fixed, m0, m1, a.ep.scale * S1,
                  a.ep.scale * S2, res);
   }
-  volume_epilogue<BLOCK, true, W3, !F32, F32>(a.ep, active, idx, a.nodes, res, a.out, blk, nblk);
+  volume_epilogue<BLOCK, true, W3, !F32>(a.ep, active, idx, a.nodes, res, a.out, blk, nblk);
 }
 
 // The same imaginary half as a persistent grid: CTA b of the grid takes the
@@ -460,7 +460,7 @@ __device__ __forceinline__ void volume_tangent_persistent(const TanVolArgs<T>& a
       if (active) {
         double res[3];
         tile_sweep<T, NS, EPB>(a, sm, le, k1, k2, idx, Da, Db, sc, S1, S2, coef32, res);
-        epilogue_node<W3, !F32, F32>(a.ep, coef, idx, a.nodes, res, a.out, da, db, dcc, dab, dbc);
+        epilogue_node<W3, !F32>(a.ep, coef, idx, a.nodes, res, a.out, da, db, dcc, dab, dbc);
       }
     }
   } else {
@@ -494,12 +494,12 @@ __device__ __forceinline__ void volume_tangent_persistent(const TanVolArgs<T>& a
         double res[3];
         fx_sweep<NS>(sm.sF[le], &sm.sB[le][0][0][0], k1, k2, sm.sD[k1], sm.sD[k2], dc, dscale, fixed, m0, m1, a.ep.scale * S1,
                      a.ep.scale * S2, res);
-        epilogue_node<W3, !F32, F32>(a.ep, coef, idx, a.nodes, res, a.out, da, db, dcc, dab, dbc);
+        epilogue_node<W3, !F32>(a.ep, coef, idx, a.nodes, res, a.out, da, db, dcc, dab, dbc);
       }
     }
   }
-  __shared__ double sred[(F32 ? 5 : 3) * BLOCK];
-  epilogue_finish<BLOCK, W3, F32>(a.ep, da, db, dcc, blockIdx.x, gridDim.x, dab, dbc, sred);
+  __shared__ double sred[(W3 ? 5 : 3) * BLOCK];
+  epilogue_finish<BLOCK, W3>(a.ep, da, db, dcc, blockIdx.x, gridDim.x, dab, dbc, sred);
 }
 
 }  // namespace swepi

@@ -232,7 +232,6 @@ __device__ __forceinline__ void tile_body(const TanVolArgs<float>& a, const DfrC
   const int t = threadIdx.x;
   const int le = t / NN, node = t % NN, k2 = node / NS, k1 = node % NS;
   double da = 0.0, db = 0.0, dcc = 0.0, dab = 0.0, dbc = 0.0;
-  const bool cd = DOTS && ep.cdot_out != nullptr;
   bool ok = true;
   int k = 0;
   for (long long tile = blockIdx.x; tile < ntiles; tile += G, ++k) {
@@ -317,12 +316,12 @@ __device__ __forceinline__ void tile_body(const TanVolArgs<float>& a, const DfrC
           if (dA) {
             const double va = sdot[(1 * 3 + mu) * TN + t];
             da = fma(o, va, da);
-            if (cd) dab = fma(vb, va, dab);
+            dab = fma(vb, va, dab);
           }
           if (dC) {
             const double vc = sdot[(0 * 3 + mu) * TN + t];
             dcc = fma(o, vc, dcc);
-            if (cd) dbc = fma(vb, vc, dbc);
+            dbc = fma(vb, vc, dbc);
           }
         }
       }
@@ -335,7 +334,7 @@ __device__ __forceinline__ void tile_body(const TanVolArgs<float>& a, const DfrC
   // waited for; after a wait that gave up the call reports SW_ETIMEOUT and its
   // result is not used): the first one holds the reduction scratch (5 TN doubles)
   static_assert(5 * TN * sizeof(double) <= L::stage, "reduction scratch larger than a stage");
-  epilogue_finish<TN, W3, true>(ep, da, db, dcc, blockIdx.x, gridDim.x, dab, dbc, reinterpret_cast<double*>(sm));
+  epilogue_finish<TN, W3>(ep, da, db, dcc, blockIdx.x, gridDim.x, dab, dbc, reinterpret_cast<double*>(sm));
 }
 
 // CTAs of the persistent grid per SM: two with the window vectors staged, three without

@@ -191,7 +191,7 @@ __device__ __forceinline__ AugEpilogue iter_epilogue(const EnsDesc& d, int j) {
   ep.skip = d.flags;
   ep.dotA = (j >= 1) ? Vi - d.ldv : nullptr;
   ep.dotB = Vi;
-  ep.cprev = d.cdot + j;
+  ep.cdot_out = d.cdot + j;
   ep.h1_out = (j >= 1) ? d.H + (long long)(j - 1) * d.ldh + j : nullptr;
   ep.h2_out = d.H + (long long)j * d.ldh + j;
   ep.dpart = d.vpart;
@@ -305,48 +305,29 @@ __device__ void update_task(const EnsDesc& d, EnsDyn& y, unsigned int local, Ens
   signal_done(&y.upd_done);
 }
 
-// V_{j+1} = z / h_{j+1,j}, V_{j+1} . V_j -> cdot[j+1]; the member's last task
-// resets the phase counters and advances its basis index
+// V_{j+1} = z / h_{j+1,j}; the member's last task resets the phase counters and
+// advances its basis index
 template <int BLOCK>
 __device__ void scale_task(const EnsDesc& d, EnsDyn& y, unsigned int local, EnsCtl* ctl, int member) {
   if (threadIdx.x == 0) wait_count(&y.upd_done, d.n_vec, ctl, 3 | (member << 4));
   __syncthreads();
   const int j = y.j;
-  const bool skip = __ldcg(d.flags) != 0;
-  const long long N = d.n + d.p;
-  double acc = 0.0;
-  __shared__ double s_r;   // one division per task (a chain of FP64 instructions)
-  if (threadIdx.x == 0) s_r = skip ? 0.0 : 1.0 / __ldcg(d.H + (long long)(j + 1) * d.ldh + j);
-  __syncthreads();
-  if (!skip) {
-    double* z = d.V + (long long)(j + 1) * d.ldv;
-    const double* VB = d.V + (long long)j * d.ldv;
-    const double r = s_r;
-    const long long i0 = (long long)local * d.vec_len, i1 = min(i0 + d.vec_len, N);
-    acc = scale_dot_range(z, VB, r, i0 + threadIdx.x, i1, BLOCK);
+  if (__ldcg(d.flags) == 0) {
+    const double r = inverse_norm(d.H + (long long)(j + 1) * d.ldh + j);
+    const long long i0 = (long long)local * d.vec_len, i1 = min(i0 + d.vec_len, d.n + d.p);
+    scale_range(d.V + (long long)(j + 1) * d.ldv, r, i0 + threadIdx.x, i1, BLOCK);
   }
-  const double b = block_sum<BLOCK>(acc);
-  __shared__ bool last;
-  if (threadIdx.x == 0) {
-    d.upart[local] = b;
-    __threadfence();
-    last = atomicAdd(&y.scl_ticket, 1u) == d.n_vec - 1;
-  }
-  __syncthreads();
-  if (!last) return;
+  __syncthreads();   // the CTA's entries are written before its ticket
+  if (threadIdx.x != 0) return;
   __threadfence();
-  double s = 0.0;
-  for (unsigned int k = threadIdx.x; k < d.n_vec; k += BLOCK) s += __ldcg(d.upart + k);
-  s = block_sum<BLOCK>(s);
-  if (threadIdx.x == 0) {
-    if (!skip) d.cdot[j + 1] = s;
-    y.face_done = 0u;
-    y.vol_done = 0u;
-    y.upd_done = 0u;
-    y.scl_ticket = 0u;
-    y.j = j + 1;
-    __threadfence();
-  }
+  if (atomicAdd(&y.scl_ticket, 1u) != d.n_vec - 1) return;
+  __threadfence();
+  y.face_done = 0u;
+  y.vol_done = 0u;
+  y.upd_done = 0u;
+  y.scl_ticket = 0u;
+  y.j = j + 1;
+  __threadfence();
 }
 
 template <int BLOCK>

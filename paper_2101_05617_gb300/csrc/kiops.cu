@@ -72,12 +72,10 @@ int ensure_krylov(Ctx& c, int m_max) {
   if (cudaMalloc(&c.d_H, sizeof(double) * c.ldh * c.ldh) != cudaSuccess) return SW_ENOMEM;
   if (cudaMalloc(&c.d_F, sizeof(double) * c.ldh * c.ldh) != cudaSuccess) return SW_ENOMEM;
   if (cudaMalloc(&c.d_expm_ws, sizeof(double) * 8 * 160 * 160) != cudaSuccess) return SW_ENOMEM;
-  if (!c.d_partials && cudaMalloc(&c.d_partials, sizeof(double) * 5 * RED_BLOCKS) != cudaSuccess) return SW_ENOMEM;
+  if (!c.d_partials && cudaMalloc(&c.d_partials, sizeof(double) * 6 * RED_BLOCKS) != cudaSuccess) return SW_ENOMEM;
   if (!c.d_vpart && cudaMalloc(&c.d_vpart, sizeof(double) * 5 * (c.nelem + 1)) != cudaSuccess) return SW_ENOMEM;
   free_ptr(c.d_cdot);
   if (cudaMalloc(&c.d_cdot, sizeof(double) * c.ldh) != cudaSuccess) return SW_ENOMEM;
-  free_ptr(c.d_cdot2);
-  if (cudaMalloc(&c.d_cdot2, sizeof(double) * c.ldh) != cudaSuccess) return SW_ENOMEM;
   if (!c.d_scal && cudaMalloc(&c.d_scal, sizeof(double) * 64) != cudaSuccess) return SW_ENOMEM;
   if (!c.d_flags) {
     if (cudaMalloc(&c.d_flags, sizeof(int) * 16) != cudaSuccess) return SW_ENOMEM;
@@ -113,8 +111,9 @@ int kiops_run(Ctx& c, const double* q_lin, double dt, double tau_out, int nb, co
     }
   }
   if (cudaMemsetAsync(c.d_flags + 3, 0, sizeof(int), s) != cudaSuccess) return SW_ECUDA;
-  // the pass and epilogue tickets, in case a wait that gave up left them mid-count
-  if (cudaMemsetAsync(c.d_flags + 8, 0, sizeof(int) * 2, s) != cudaSuccess) return SW_ECUDA;
+  // the pass and epilogue tickets and the cooperative passes' barrier counter, in
+  // case a wait that gave up left them mid-count
+  if (cudaMemsetAsync(c.d_flags + 8, 0, sizeof(int) * 3, s) != cudaSuccess) return SW_ECUDA;
   // X = [b_0; 0 .. 0 mu]
   if (bk[0]) {
     if (cudaMemcpyAsync(c.d_X, bk[0], sizeof(double) * n, cudaMemcpyDeviceToDevice, s) != cudaSuccess) return SW_ECUDA;
@@ -221,12 +220,10 @@ int kiops_run(Ctx& c, const double* q_lin, double dt, double tau_out, int nb, co
         const double* wA = (it >= 1) ? V + (it - 1) * ldv : nullptr;
         const double* wC = hC ? V + (it - 2) * ldv : nullptr;
         // complex64-bulk form: the FP32 volume kernel forms no dots; a pass of
-        // their own (orth_dots_dev) takes them and the V . V products
+        // their own (orth_dots_dev) takes them
         ep.dotA = use32 ? nullptr : wA;
         ep.dotB = use32 ? nullptr : Vi;
         ep.dotC = use32 ? nullptr : wC;
-        ep.cprev = c.d_cdot + it;
-        ep.cprevC = c.d_cdot2 + it;
         ep.cprevAC = (it >= 1) ? c.d_cdot + it - 1 : nullptr;
         ep.h0_out = hC;
         ep.h1_out = hA;
@@ -235,39 +232,34 @@ int kiops_run(Ctx& c, const double* q_lin, double dt, double tau_out, int nb, co
         ep.dticket = (unsigned int*)(c.d_flags + 9);
         ep.n = n;
         ep.v32 = use32 ? c.d_V32 + it * ldv : nullptr;
-        ep.cdot_out = ep.cdot2_out = nullptr;
+        ep.cdot_out = c.d_cdot + it;
         rc = use_lin ? launch_jvp_lin(c, Vi, Vn, ep, s, c.jvp_mode == 2) : launch_jvp(c, q_lin, Vi, kEpsJvp, Vn, ep, s);
         if (rc) return rc;
         double* hs = c.d_H + (long long)(it + 1) * c.ldh + it;
         if (use32) {
           double* cd = wA ? c.d_cdot + it : nullptr;
-          double* cd2 = wC ? c.d_cdot2 + it : nullptr;
           const double* cpac = wC ? c.d_cdot + it - 1 : nullptr;
           float* z32 = c.d_V32 + (it + 1) * ldv;
           if (fused) {
-            rc = launch_orth3_fused(c, Vn, wA, Vi, wC, N, o.tol, it + 1, hC, hA, hB, hs, cd, cd2, cpac, z32, s);
-          } else if (!(rc = launch_orth_dots(c, Vn, Vi, wA, wC, N, hC, hA, hB, cd, cd2, cpac, s)) &&
-                     !(rc = launch_update_norm(c, Vn, wA, Vi, hA, hB, N, hs, o.tol, it + 1, s, wC, hC))) {
-            rc = launch_scale_dot(c, Vn, Vi, hs, N, nullptr, s, nullptr, nullptr, z32);
+            rc = launch_orth3_fused(c, Vn, wA, Vi, wC, N, o.tol, it + 1, hC, hA, hB, hs, cd, cpac, z32, s);
+          } else if (!(rc = launch_orth_dots(c, Vn, Vi, wA, wC, N, hC, hA, hB, cd, cpac, s)) &&
+                     !(rc = launch_update_norm(c, Vn, wA, Vi, hA, hB, N, hs, o.tol, it + 1, red_blocks(N), s, wC, hC))) {
+            rc = launch_scale(c, Vn, hs, N, red_blocks(N), s, z32);
           }
           if (rc) return rc;
           continue;
         }
-        // V_{j+1} . V_{j-1} is needed by the window of three two iterations later
-        const double* Vprev = (o.iop == 3 && it >= 1) ? V + (it - 1) * ldv : nullptr;
-        double* cn = c.d_cdot + it + 1;
         if (fused) {
-          rc = launch_orth_fused(c, Vn, wA, Vi, hA, hB, N, hs, o.tol, it + 1, wC, hC, cn, Vprev,
-                                 c.d_cdot2 + it + 1, nullptr, s);
-        } else if (!(rc = launch_update_norm(c, Vn, wA, Vi, hA, hB, N, hs, o.tol, it + 1, s, wC, hC))) {
-          rc = launch_scale_dot(c, Vn, Vi, hs, N, cn, s, Vprev, c.d_cdot2 + it + 1, nullptr);
+          rc = launch_orth_fused(c, Vn, wA, Vi, hA, hB, N, hs, o.tol, it + 1, wC, hC, s);
+        } else if (!(rc = launch_update_norm(c, Vn, wA, Vi, hA, hB, N, hs, o.tol, it + 1, orth_blocks(N), s,
+                                              wC, hC))) {
+          rc = launch_scale(c, Vn, hs, N, orth_blocks(N), s);
         }
         if (rc) return rc;
         continue;
       }
       ep.dotA = ep.dotB = ep.dotC = nullptr;
       ep.v32 = nullptr;
-      ep.cdot_out = ep.cdot2_out = nullptr;
       rc = use_lin ? launch_jvp_lin(c, Vi, Vn, ep, s, c.jvp_mode == 2) : launch_jvp(c, q_lin, Vi, kEpsJvp, Vn, ep, s);
       if (rc) return rc;
       for (int i = std::max(0, it - o.iop + 1); i <= it; ++i) {

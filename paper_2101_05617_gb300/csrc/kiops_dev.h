@@ -40,7 +40,6 @@ struct KFix {
   int* flags;
   double* scal;
   double* cdot;
-  double* cdot2;
   double* vpart;
   double* partials;
   double* ws;         // exponential workspace
@@ -68,8 +67,6 @@ __device__ __forceinline__ void iter_epilogue_dev(AugEpilogue& ep, const KDev& k
   ep.dotA = (!sep && it >= 1) ? Vi - f.ldv : nullptr;
   ep.dotB = sep ? nullptr : Vi;
   ep.dotC = (!sep && w3 && it >= 2) ? Vi - 2 * f.ldv : nullptr;
-  ep.cprev = f.cdot + it;
-  ep.cprevC = f.cdot2 + it;
   ep.cprevAC = (it >= 1) ? f.cdot + it - 1 : nullptr;
   ep.h0_out = (w3 && it >= 2) ? f.H + (long long)(it - 2) * f.ldh + it : nullptr;
   ep.h1_out = (it >= 1) ? f.H + (long long)(it - 1) * f.ldh + it : nullptr;
@@ -78,7 +75,7 @@ __device__ __forceinline__ void iter_epilogue_dev(AugEpilogue& ep, const KDev& k
   ep.dticket = reinterpret_cast<unsigned int*>(f.flags + 9);
   ep.n = f.n;
   ep.v32 = sep ? f.V32 + (long long)it * f.ldv : nullptr;
-  ep.cdot_out = ep.cdot2_out = nullptr;
+  ep.cdot_out = f.cdot + it;
 }
 #endif
 

@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kRedThreads) kg_dots_kernel(const KDev* __rest
   double* hB = f.H + (long long)it * f.ldh + it;
   double* hC = (W3 && it >= 2) ? f.H + (long long)(it - 2) * f.ldh + it : nullptr;
   orth_dots_dev(Vn, Vi, VA, VC, f.N, f.partials, reinterpret_cast<unsigned int*>(f.flags + 8), f.flags, hC, hA, hB,
-                VA ? f.cdot + it : nullptr, VC ? f.cdot2 + it : nullptr, VC ? f.cdot + it - 1 : nullptr);
+                VA ? f.cdot + it : nullptr, VC ? f.cdot + it - 1 : nullptr);
 }
 
 template <bool W3>
@@ -160,17 +160,11 @@ __global__ void __launch_bounds__(kRedThreads) kg_update_kernel(const KDev* __re
                   f.flags, it + 1, VC, hC);
 }
 
-template <bool W3>
 __global__ void __launch_bounds__(kRedThreads) kg_scale_kernel(const KDev* __restrict__ kd, KFix f) {
   const int it = kd->it;
-  double* Vi = f.V + (long long)it * f.ldv;
-  double* Vn = Vi + f.ldv;
+  double* Vn = f.V + (long long)(it + 1) * f.ldv;
   const double* hs = f.H + (long long)(it + 1) * f.ldh + it;
-  const double* Vprev = (W3 && it >= 1) ? Vi - f.ldv : nullptr;
-  float* z32 = f.V32 ? f.V32 + (long long)(it + 1) * f.ldv : nullptr;
-  // complex64-bulk form (FP32 basis copy): the next volume kernel forms the V . V dots
-  scale_dot_dev(Vn, Vi, hs, f.N, f.partials, reinterpret_cast<unsigned int*>(f.flags + 8),
-                f.V32 ? nullptr : f.cdot + it + 1, f.flags, Vprev, f.cdot2 + it + 1, z32);
+  scale_dev(Vn, hs, f.N, f.flags, f.V32 ? f.V32 + (long long)(it + 1) * f.ldv : nullptr);
 }
 
 __global__ void kg_advance_kernel(KDev* kd, KFix f, cudaGraphConditionalHandle hi) {
@@ -338,7 +332,6 @@ KFix make_fix(const Ctx& c, int p, bool fp32) {
   f.flags = c.d_flags;
   f.scal = c.d_scal;
   f.cdot = c.d_cdot;
-  f.cdot2 = c.d_cdot2;
   f.vpart = c.d_vpart;
   f.partials = c.d_partials;
   f.ws = c.d_expm_ws;
@@ -390,12 +383,13 @@ int build(Ctx& c, KGraph& G, int p, int iop, bool fp32, int mmax) {
       else
         kg_dots_kernel<false><<<red_blocks(f.N), kRedThreads, 0, s>>>(kd, f);
     }
+    const int ob = f.V32 ? red_blocks(f.N) : orth_blocks(f.N);   // as the host driver's passes
     if (w3) {
-      kg_update_kernel<true><<<red_blocks(f.N), kRedThreads, 0, s>>>(kd, f);
-      kg_scale_kernel<true><<<red_blocks(f.N), kRedThreads, 0, s>>>(kd, f);
+      kg_update_kernel<true><<<ob, kRedThreads, 0, s>>>(kd, f);
+      kg_scale_kernel<<<ob, kRedThreads, 0, s>>>(kd, f);
     } else {
-      kg_update_kernel<false><<<red_blocks(f.N), kRedThreads, 0, s>>>(kd, f);
-      kg_scale_kernel<false><<<red_blocks(f.N), kRedThreads, 0, s>>>(kd, f);
+      kg_update_kernel<false><<<ob, kRedThreads, 0, s>>>(kd, f);
+      kg_scale_kernel<<<ob, kRedThreads, 0, s>>>(kd, f);
     }
     kg_advance_kernel<<<1, 1, 0, s>>>(kd, f, hi);
     return cuda_status(cudaGetLastError());

@@ -156,46 +156,41 @@ __global__ void __launch_bounds__(RED_THREADS) update_norm_kernel(double* __rest
   update_norm_dev(z, VA, VB, h1p, h2p, n, partials, ticket, hsub, tol, happy, happy_value, VC, h0p);
 }
 
-__global__ void __launch_bounds__(RED_THREADS) scale_dot_kernel(double* __restrict__ z, const double* __restrict__ VB,
-                                                                const double* hsub, long long n, double* partials,
-                                                                unsigned int* ticket, double* c_out, const int* happy,
-                                                                const double* __restrict__ VA, double* c2_out,
-                                                                float* __restrict__ z32) {
+__global__ void __launch_bounds__(RED_THREADS) scale_kernel(double* __restrict__ z, const double* hsub, long long n,
+                                                            const int* happy, float* __restrict__ z32) {
   pdl_wait();
   pdl_trigger();
-  scale_dot_dev(z, VB, hsub, n, partials, ticket, c_out, happy, VA, c2_out, z32);
+  scale_dev(z, hsub, n, happy, z32);
 }
 
 // both passes in one cooperative launch (orth_fused_dev)
-__global__ void __launch_bounds__(RED_THREADS, 4) orth_fused_kernel(
+__global__ void __launch_bounds__(RED_THREADS, 2) orth_fused_kernel(
     double* __restrict__ z, const double* __restrict__ VA, const double* __restrict__ VB, const double* h1p,
-    const double* h2p, long long n, double* partials, unsigned int* ticket, double* hsub, double tol, int* happy,
-    int happy_value, const double* __restrict__ VC, const double* h0p, double* c_out, const double* __restrict__ VA2,
-    double* c2_out, float* __restrict__ z32, unsigned int* gen, int* err) {
+    const double* h2p, long long n, double* partials, double* hsub, double tol, int* happy, int happy_value,
+    const double* __restrict__ VC, const double* h0p, unsigned int* bar, int* err) {
   pdl_trigger();
-  orth_fused_dev(z, VA, VB, h1p, h2p, n, partials, ticket, hsub, tol, happy, happy_value, VC, h0p, c_out, VA2, c2_out,
-                 z32, gen, err);
+  orth_fused_dev(z, VA, VB, h1p, h2p, n, partials, hsub, tol, happy, happy_value, VC, h0p, bar, err);
 }
 
 // the dot pass of the complex64-bulk form (orth_dots_dev)
 __global__ void __launch_bounds__(RED_THREADS) orth_dots_kernel(
     const double* __restrict__ z, const double* __restrict__ VB, const double* __restrict__ VA,
     const double* __restrict__ VC, long long n, double* partials, unsigned int* ticket, const int* happy,
-    double* h0_out, double* h1_out, double* h2_out, double* cdot_out, double* cdot2_out, const double* cprevAC) {
+    double* h0_out, double* h1_out, double* h2_out, double* cdot_out, const double* cprevAC) {
   pdl_wait();
   pdl_trigger();
-  orth_dots_dev(z, VB, VA, VC, n, partials, ticket, happy, h0_out, h1_out, h2_out, cdot_out, cdot2_out, cprevAC);
+  orth_dots_dev(z, VB, VA, VC, n, partials, ticket, happy, h0_out, h1_out, h2_out, cdot_out, cprevAC);
 }
 
 // the dot, update and scale passes in one cooperative launch (orth3_fused_dev)
 __global__ void __launch_bounds__(RED_THREADS, 4) orth3_fused_kernel(
     double* __restrict__ z, const double* __restrict__ VA, const double* __restrict__ VB,
     const double* __restrict__ VC, long long n, double* partials, unsigned int* ticket, double tol, int* happy,
-    int happy_value, double* h0p, double* h1p, double* h2p, double* hsub, double* cdot_out, double* cdot2_out,
-    const double* cprevAC, float* __restrict__ z32, unsigned int* gen, int* err) {
+    int happy_value, double* h0p, double* h1p, double* h2p, double* hsub, double* cdot_out, const double* cprevAC,
+    float* __restrict__ z32, unsigned int* gen, int* err) {
   pdl_trigger();
   orth3_fused_dev(z, VA, VB, VC, n, partials, ticket, tol, happy, happy_value, h0p, h1p, h2p, hsub, cdot_out,
-                  cdot2_out, cprevAC, z32, gen, err);
+                  cprevAC, z32, gen, err);
 }
 
 int blocks_for(long long n, int threads) {
@@ -288,15 +283,15 @@ int launch_scale_inv(Ctx& c, double* y, const double* x, const double* s_dev, lo
 }
 
 int launch_update_norm(Ctx& c, double* z, const double* VA, const double* VB, const double* h1, const double* h2,
-                       long long N, double* hsub, double tol, int happy_value, cudaStream_t s, const double* VC,
-                       const double* h0) {
+                       long long N, double* hsub, double tol, int happy_value, int blocks, cudaStream_t s,
+                       const double* VC, const double* h0) {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (prof_on(c, PK_ORTH)) {
     e0 = prof_event(c);
     e1 = prof_event(c);
     cudaEventRecord(e0, s);
   }
-  if (launch_pdl(update_norm_kernel, dim3(red_blocks(N)), dim3(RED_THREADS), s, z, VA, VB, h1, h2, N, c.d_partials,
+  if (launch_pdl(update_norm_kernel, dim3(blocks), dim3(RED_THREADS), s, z, VA, VB, h1, h2, N, c.d_partials,
                  (unsigned int*)(c.d_flags + 8), hsub, tol, c.d_flags, happy_value, VC, h0) != cudaSuccess)
     return SW_ECUDA;
   if (prof_on(c, PK_ORTH)) {
@@ -307,16 +302,15 @@ int launch_update_norm(Ctx& c, double* z, const double* VA, const double* VB, co
   return cuda_status(cudaGetLastError());
 }
 
-int launch_scale_dot(Ctx& c, double* z, const double* VB, const double* hsub, long long N, double* c_out,
-                     cudaStream_t s, const double* VA, double* c2_out, float* z32) {
+int launch_scale(Ctx& c, double* z, const double* hsub, long long N, int blocks, cudaStream_t s, float* z32) {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (prof_on(c, PK_ORTH)) {
     e0 = prof_event(c);
     e1 = prof_event(c);
     cudaEventRecord(e0, s);
   }
-  if (launch_pdl(scale_dot_kernel, dim3(red_blocks(N)), dim3(RED_THREADS), s, z, VB, hsub, N, c.d_partials,
-                 (unsigned int*)(c.d_flags + 8), c_out, c.d_flags, VA, c2_out, z32) != cudaSuccess)
+  if (launch_pdl(scale_kernel, dim3(blocks), dim3(RED_THREADS), s, z, hsub, N,
+                 static_cast<const int*>(c.d_flags), z32) != cudaSuccess)
     return SW_ECUDA;
   if (prof_on(c, PK_ORTH)) {
     cudaEventRecord(e1, s);
@@ -335,15 +329,15 @@ int orth_fused_available(Ctx& c) {
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c.device) == cudaSuccess &&
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, orth_fused_kernel, RED_THREADS, 0) == cudaSuccess &&
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb3, orth3_fused_kernel, RED_THREADS, 0) == cudaSuccess &&
-        (long long)nb * sms >= RED_BLOCKS && (long long)nb3 * sms >= RED_BLOCKS)
+        (long long)nb * sms >= ORTH_BLOCKS && (long long)nb3 * sms >= RED_BLOCKS)
       c.orth_fused = 1;
   }
   return c.orth_fused > 0;
 }
 
 int launch_orth_dots(Ctx& c, const double* z, const double* VB, const double* VA, const double* VC, long long N,
-                     double* h0_out, double* h1_out, double* h2_out, double* cdot_out, double* cdot2_out,
-                     const double* cprevAC, cudaStream_t s) {
+                     double* h0_out, double* h1_out, double* h2_out, double* cdot_out, const double* cprevAC,
+                     cudaStream_t s) {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (prof_on(c, PK_ORTH)) {
     e0 = prof_event(c);
@@ -352,7 +346,7 @@ int launch_orth_dots(Ctx& c, const double* z, const double* VB, const double* VA
   }
   if (launch_pdl(orth_dots_kernel, dim3(red_blocks(N)), dim3(RED_THREADS), s, z, VB, VA, VC, N, c.d_partials,
                  reinterpret_cast<unsigned int*>(c.d_flags + 8), static_cast<const int*>(c.d_flags), h0_out, h1_out,
-                 h2_out, cdot_out, cdot2_out, cprevAC) != cudaSuccess)
+                 h2_out, cdot_out, cprevAC) != cudaSuccess)
     return SW_ECUDA;
   if (prof_on(c, PK_ORTH)) {
     cudaEventRecord(e1, s);
@@ -364,7 +358,7 @@ int launch_orth_dots(Ctx& c, const double* z, const double* VB, const double* VA
 
 int launch_orth3_fused(Ctx& c, double* z, const double* VA, const double* VB, const double* VC, long long N,
                        double tol, int happy_value, double* h0p, double* h1p, double* h2p, double* hsub,
-                       double* cdot_out, double* cdot2_out, const double* cprevAC, float* z32, cudaStream_t s) {
+                       double* cdot_out, const double* cprevAC, float* z32, cudaStream_t s) {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (prof_on(c, PK_ORTH)) {
     e0 = prof_event(c);
@@ -382,7 +376,7 @@ int launch_orth3_fused(Ctx& c, double* z, const double* VA, const double* VB, co
   cfg.numAttrs = 1;
   if (cudaLaunchKernelEx(&cfg, orth3_fused_kernel, z, VA, VB, VC, N, c.d_partials,
                          reinterpret_cast<unsigned int*>(c.d_flags + 8), tol, c.d_flags, happy_value, h0p, h1p, h2p,
-                         hsub, cdot_out, cdot2_out, cprevAC, z32, reinterpret_cast<unsigned int*>(c.d_flags + 10),
+                         hsub, cdot_out, cprevAC, z32, reinterpret_cast<unsigned int*>(c.d_flags + 10),
                          c.d_flags + 3) != cudaSuccess)
     return SW_ECUDA;
   if (prof_on(c, PK_ORTH)) {
@@ -396,7 +390,7 @@ int launch_orth3_fused(Ctx& c, double* z, const double* VA, const double* VB, co
 
 int launch_orth_fused(Ctx& c, double* z, const double* VA, const double* VB, const double* h1, const double* h2,
                       long long N, double* hsub, double tol, int happy_value, const double* VC, const double* h0,
-                      double* c_out, const double* VA2, double* c2_out, float* z32, cudaStream_t s) {
+                      cudaStream_t s) {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (prof_on(c, PK_ORTH)) {
     e0 = prof_event(c);
@@ -404,7 +398,7 @@ int launch_orth_fused(Ctx& c, double* z, const double* VA, const double* VB, con
     cudaEventRecord(e0, s);
   }
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(red_blocks(N));
+  cfg.gridDim = dim3(orth_blocks(N));
   cfg.blockDim = dim3(RED_THREADS);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
@@ -412,10 +406,8 @@ int launch_orth_fused(Ctx& c, double* z, const double* VA, const double* VB, con
   at[0].val.cooperative = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, orth_fused_kernel, z, VA, VB, h1, h2, N, c.d_partials,
-                         reinterpret_cast<unsigned int*>(c.d_flags + 8), hsub, tol, c.d_flags, happy_value, VC, h0,
-                         c_out, VA2, c2_out, z32, reinterpret_cast<unsigned int*>(c.d_flags + 10),
-                         c.d_flags + 3) != cudaSuccess)
+  if (cudaLaunchKernelEx(&cfg, orth_fused_kernel, z, VA, VB, h1, h2, N, c.d_partials, hsub, tol, c.d_flags, happy_value, VC, h0,
+                         reinterpret_cast<unsigned int*>(c.d_flags + 10), c.d_flags + 3) != cudaSuccess)
     return SW_ECUDA;
   if (prof_on(c, PK_ORTH)) {
     cudaEventRecord(e1, s);

@@ -89,9 +89,8 @@ template <bool HA, bool HC>
 __device__ __forceinline__ double mgs_update_range_t(double* __restrict__ z, const double* __restrict__ VA,
                                                      const double* __restrict__ VB, double h1, double h2, long long i,
                                                      long long i1, long long stride, const double* __restrict__ VC,
-                                                     double h0) {
+                                                     double h0, double acc = 0.0) {
     constexpr int D = HC ? 4 : 8;   // entries in flight per thread
-  double acc = 0.0;
   for (; i + (D - 1) * stride < i1; i += D * stride) {
     double v[D], b[D], a[D], c[D];
 #pragma unroll
@@ -147,97 +146,127 @@ __device__ __forceinline__ double mgs_update_range(double* __restrict__ z, const
             : mgs_update_range_t<false, false>(z, VA, VB, h1, h2, i, i1, stride, VC, h0);
 }
 
-//   z *= r; returns the thread's sum of z_i VB_i, and with VA also the sum of
-//   z_i VA_i in *za; with z32, also the FP32 copy of the scaled z (rounded to
-//   nearest) for the complex64-bulk form's kernels
-__device__ __forceinline__ double scale_dot_range(double* __restrict__ z, const double* __restrict__ VB, double r,
-                                                  long long i, long long i1, long long stride,
-                                                  const double* __restrict__ VA = nullptr, double* za = nullptr,
-                                                  float* __restrict__ z32 = nullptr) {
-  if (VA) {
-    double acc = 0.0, acc2 = 0.0;
-    for (; i + 3 * stride < i1; i += 4 * stride) {
-      double v[4], b[4], a[4];
+//   z *= r; with z32, also the FP32 copy of the scaled z (rounded to nearest)
+//   for the complex64-bulk form's kernels; eight entries in flight, the last
+//   batch guarded
+__device__ __forceinline__ void scale_range(double* __restrict__ z, double r, long long i, long long i1,
+                                            long long stride, float* __restrict__ z32 = nullptr) {
+  constexpr int D = 8;
+  for (; i < i1; i += D * stride) {
+    double v[D];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        v[k] = __ldcg(z + i + k * stride);
-        b[k] = VB[i + k * stride];
-        a[k] = VA[i + k * stride];
-      }
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        v[k] *= r;
-        z[i + k * stride] = v[k];
-        if (z32) z32[i + k * stride] = f64_to_f32_bits(v[k]);
-        acc = fma(v[k], b[k], acc);
-        acc2 = fma(v[k], a[k], acc2);
-      }
+    for (int k = 0; k < D; ++k) {
+      const long long j = i + k * stride;
+      if (j < i1) v[k] = __ldcg(z + j);
     }
-    if (i < i1) {
-      double v[3], b[3], a[3];
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const long long j = i + k * stride;
-        if (j >= i1) break;
-        v[k] = __ldcg(z + j);
-        b[k] = VB[j];
-        a[k] = VA[j];
-      }
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const long long j = i + k * stride;
-        if (j >= i1) break;
+    for (int k = 0; k < D; ++k) {
+      const long long j = i + k * stride;
+      if (j < i1) {
         v[k] *= r;
         z[j] = v[k];
         if (z32) z32[j] = f64_to_f32_bits(v[k]);
-        acc = fma(v[k], b[k], acc);
-        acc2 = fma(v[k], a[k], acc2);
       }
     }
-    *za = acc2;
-    return acc;
   }
+}
+
+// The first K entries of a thread (indices i0, i0 + stride, ...) kept in
+// registers from one phase of a fused pass to the next, instead of through
+// memory; the entries past them take the memory path.  K = 32 covers every
+// entry up to 2.49 M unknowns (6 x 60 x 60, p = 5: 30 a thread).
+constexpr int kKeep = 32;
+
+// mgs_update_range_t with the kept entries' z in registers; they are not stored.
+// The same operations in the same order as mgs_update_range_t.
+// The next batch of D entries is on its way while one is computed (two CTAs an
+// SM leave few other warps to hide a load behind).
+template <bool HA, bool HC>
+__device__ __forceinline__ double mgs_update_keep_t(double* __restrict__ z, const double* __restrict__ VA,
+                                                    const double* __restrict__ VB, double h1, double h2, long long i0,
+                                                    long long i1, long long stride, const double* __restrict__ VC,
+                                                    double h0, double (&keep)[kKeep]) {
+  constexpr int D = HC ? 2 : 4;
   double acc = 0.0;
-  for (; i + 3 * stride < i1; i += 4 * stride) {
-    double v[4], b[4];
+  double b[2][D], a[2][D], c[2][D];
+  auto load = [&](int q, int s) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      v[k] = __ldcg(z + i + k * stride);
-      b[k] = VB[i + k * stride];
+    for (int k = 0; k < D; ++k) {
+      const long long j = i0 + (q + k) * stride;
+      if (j < i1) {
+        keep[q + k] = __ldcg(z + j);
+        b[s][k] = VB[j];
+        if (HA) a[s][k] = VA[j];
+        if (HC) c[s][k] = VC[j];
+      }
     }
+  };
+  load(0, 0);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      v[k] *= r;
-      z[i + k * stride] = v[k];
-      if (z32) z32[i + k * stride] = f64_to_f32_bits(v[k]);
-      acc = fma(v[k], b[k], acc);
-    }
-  }
-  if (i < i1) {
-    double v[3], b[3];
+  for (int q = 0; q < kKeep; q += D) {
+    if (i0 + q * stride >= i1) break;   // a guarded-off FP64 instruction would still take the pipe
+    const int s = (q / D) & 1;
+    if (q + D < kKeep) load(q + D, s ^ 1);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const long long j = i + k * stride;
-      if (j >= i1) break;
-      v[k] = __ldcg(z + j);
-      b[k] = VB[j];
-    }
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const long long j = i + k * stride;
-      if (j >= i1) break;
-      v[k] *= r;
-      z[j] = v[k];
-      if (z32) z32[j] = f64_to_f32_bits(v[k]);
-      acc = fma(v[k], b[k], acc);
+    for (int k = 0; k < D; ++k) {
+      if (i0 + (q + k) * stride < i1) {
+        double v = keep[q + k];
+        if (HC) v = fma(-h0, c[s][k], v);
+        if (HA) v = fma(-h1, a[s][k], v);
+        v = fma(-h2, b[s][k], v);
+        keep[q + k] = v;
+        acc = fma(v, v, acc);
+      }
     }
   }
-  return acc;
+  const long long i = i0 + kKeep * stride;
+  return i < i1 ? mgs_update_range_t<HA, HC>(z, VA, VB, h1, h2, i, i1, stride, VC, h0, acc) : acc;
+}
+
+__device__ __forceinline__ double mgs_update_keep(double* __restrict__ z, const double* __restrict__ VA,
+                                                  const double* __restrict__ VB, double h1, double h2, long long i0,
+                                                  long long i1, long long stride, const double* __restrict__ VC,
+                                                  double h0, double (&keep)[kKeep]) {
+  // V_{j-2} only ever comes with V_{j-1}
+  if (VC) return mgs_update_keep_t<true, true>(z, VA, VB, h1, h2, i0, i1, stride, VC, h0, keep);
+  return VA ? mgs_update_keep_t<true, false>(z, VA, VB, h1, h2, i0, i1, stride, VC, h0, keep)
+            : mgs_update_keep_t<false, false>(z, VA, VB, h1, h2, i0, i1, stride, VC, h0, keep);
+}
+
+// scale_range with the kept entries from registers
+__device__ __forceinline__ void scale_keep(double* __restrict__ z, double r, long long i0, long long i1,
+                                           long long stride, const double (&keep)[kKeep], float* __restrict__ z32) {
+#pragma unroll
+  for (int k = 0; k < kKeep; ++k) {
+    const long long j = i0 + k * stride;
+    if (j >= i1) break;
+    const double v = keep[k] * r;
+    z[j] = v;
+    if (z32) z32[j] = f64_to_f32_bits(v);
+  }
+  const long long i = i0 + kKeep * stride;
+  if (i < i1) scale_range(z, r, i, i1, stride, z32);
 }
 
 // The two vector passes of the fused incomplete orthogonalisation, as device
 // functions of a whole grid (the stream kernels of krylov.cu and the
 // device-driven solver call them).
+// the sum over the grid's per-CTA partials in index order of the threads
+// (valid in thread 0)
+__device__ __forceinline__ double partials_sum(const double* partials) {
+  double sum = 0.0;
+  for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) sum += __ldcg(partials + i);
+  return block_sum(sum);
+}
+// ||z||_2 -> *hsub, with the happy-breakdown flag below tol (one thread)
+__device__ __forceinline__ void norm_publish(double r, double* hsub, double tol, int* happy, int happy_value) {
+  *hsub = r;
+  if (r < tol) {
+    happy[0] = 1;
+    happy[1] = happy_value;
+  }
+}
+
 // z -= h0 V_C + h1 V_A + h2 V_B (the modified Gram-Schmidt updates, oldest
 // first; V_C, V_A may be absent), then ||z||_2 -> *hsub with the
 // happy-breakdown flag below tol.  Returns 0 when the basis had already broken
@@ -263,134 +292,112 @@ __device__ __forceinline__ int update_norm_dev(double* __restrict__ z, const dou
   __syncthreads();
   if (!last) return 1;
   __threadfence();
-  double sum = 0.0;
-  for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) sum += __ldcg(partials + i);
-  sum = block_sum(sum);
+  const double sum = partials_sum(partials);
   if (threadIdx.x == 0) {
-    const double r = sqrt(sum);
-    *hsub = r;
-    if (r < tol) {
-      happy[0] = 1;
-      happy[1] = happy_value;
-    }
+    norm_publish(sqrt(sum), hsub, tol, happy, happy_value);
     *ticket = 0u;
   }
   return 2;
 }
 
-// V_next = z / *hsub in place, V_next . V_B -> *c_out and, with V_A, V_next .
-// V_A -> *c2_out (used by the next iterations' orthogonalisation); with z32
-// also the FP32 copy of V_next
-__device__ __forceinline__ void scale_dot_dev(double* __restrict__ z, const double* __restrict__ VB,
-                                              const double* hsub, long long n, double* partials, unsigned int* ticket,
-                                              double* c_out, const int* happy, const double* __restrict__ VA,
-                                              double* c2_out, float* __restrict__ z32) {
-  // through L2: in the fused launch another CTA has just written them
-  if (__ldcg(happy)) return;
-  // one division per CTA: a reciprocal is a chain of FP64 instructions, and in
-  // every warp it held the pipe as long as the pass's own work on small grids
+// 1 / *hsub, one division per CTA: a reciprocal is a chain of FP64
+// instructions, and in every warp it held the pipe as long as the pass's own
+// work on small grids (through L2: in a fused launch another CTA has just
+// written *hsub)
+__device__ __forceinline__ double inverse_norm(const double* hsub) {
   __shared__ double s_r;
   if (threadIdx.x == 0) s_r = 1.0 / __ldcg(hsub);
   __syncthreads();
-  const double r = s_r;
-  if (!c_out) {   // scale only (the next volume kernel forms the dots)
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    constexpr int D = 8;   // entries in flight per thread, the last batch guarded
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += D * stride) {
-      double v[D];
-#pragma unroll
-      for (int k = 0; k < D; ++k) {
-        const long long j = i + k * stride;
-        if (j < n) v[k] = __ldcg(z + j);
-      }
-#pragma unroll
-      for (int k = 0; k < D; ++k) {
-        const long long j = i + k * stride;
-        if (j < n) {
-          v[k] *= r;
-          z[j] = v[k];
-          if (z32) z32[j] = f64_to_f32_bits(v[k]);
-        }
-      }
-    }
-    return;
-  }
-  double acc2 = 0.0;
-  const double acc = scale_dot_range(z, VB, r, (long long)blockIdx.x * blockDim.x + threadIdx.x, n,
-                                     (long long)gridDim.x * blockDim.x, VA, &acc2, z32);
-  const double b = block_sum(acc);
-  const double b2 = VA ? block_sum(acc2) : 0.0;   // uniform condition
-  __shared__ bool last;
-  if (threadIdx.x == 0) {
-    partials[2 * blockIdx.x] = b;
-    partials[2 * blockIdx.x + 1] = b2;
-    __threadfence();
-    last = (atomicAdd(ticket, 1u) == gridDim.x - 1);
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  double sum = 0.0, sum2 = 0.0;
-  for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
-    sum += __ldcg(partials + 2 * i);
-    if (VA) sum2 += __ldcg(partials + 2 * i + 1);
-  }
-  sum = block_sum(sum);
-  if (VA) sum2 = block_sum(sum2);
-  if (threadIdx.x == 0) {
-    *c_out = sum;
-    if (VA) *c2_out = sum2;
-    *ticket = 0u;
-  }
+  return s_r;
+}
+
+// V_next = z / *hsub in place; with z32 also the FP32 copy of V_next
+__device__ __forceinline__ void scale_dev(double* __restrict__ z, const double* hsub, long long n, const int* happy,
+                                          float* __restrict__ z32) {
+  if (__ldcg(happy)) return;
+  scale_range(z, inverse_norm(hsub), (long long)blockIdx.x * blockDim.x + threadIdx.x, n,
+              (long long)gridDim.x * blockDim.x, z32);
 }
 
 // polls of the fused pass's grid-wide wait (each after a short sleep: about a
 // second in all) before it gives up
 constexpr unsigned int kOrthWaitPolls = 1u << 23;
 
-// Both passes in one launch of a grid whose CTAs are all resident at once (a
-// cooperative launch): the update pass, then -- once the CTA that finished it
-// last has published ||z|| by advancing the counter *gen -- the scale pass.
-// The same arithmetic in the same order as update_norm_dev followed by
-// scale_dot_dev on the same grid (bitwise the same results); it saves the
-// second launch and its ramp.  A CTA that waits past the bound sets *err and
-// leaves its share of the scale pass undone (the caller reports a timeout).
-__device__ __forceinline__ void orth_fused_dev(double* __restrict__ z, const double* __restrict__ VA,
-                                               const double* __restrict__ VB, const double* h1p, const double* h2p,
-                                               long long n, double* partials, unsigned int* ticket, double* hsub,
-                                               double tol, int* happy, int happy_value, const double* __restrict__ VC,
-                                               const double* h0p, double* c_out, const double* __restrict__ VA2,
-                                               double* c2_out, float* __restrict__ z32, unsigned int* gen, int* err) {
-  __shared__ unsigned int g0;
+// Barrier over the CTAs of a cooperative launch (every thread calls it; what a
+// CTA wrote before it is visible to all after it, read through L2).  The
+// counter's top bit flips when every CTA has arrived, whatever the grid: CTA 0
+// adds what is missing to 2^31, the others one each.  The wait is bounded;
+// false when it gave up (*err is set and the CTA leaves its remaining phases
+// undone; the caller's next phi-function call clears the counter).
+__device__ __forceinline__ bool grid_barrier(unsigned int* bar, int* err) {
   __shared__ int gave_up;
-  // read before this CTA's ticket (ordered by the fence ahead of it): the
-  // counter can only advance after every CTA has taken its ticket
+  __syncthreads();
   if (threadIdx.x == 0) {
-    g0 = *reinterpret_cast<volatile unsigned int*>(gen);
     gave_up = 0;
-  }
-  const int st = update_norm_dev(z, VA, VB, h1p, h2p, n, partials, ticket, hsub, tol, happy, happy_value, VC, h0p);
-  if (st == 0) return;   // uniform over the grid
-  if (threadIdx.x == 0) {
-    if (st == 2) {
-      __threadfence();
-      atomicAdd(gen, 1u);
-    } else {
-      unsigned int polls = 0;
-      while (*reinterpret_cast<volatile unsigned int*>(gen) == g0) {
-        if (++polls > kOrthWaitPolls) {
-          gave_up = 1;
-          atomicExch(err, 1);
-          break;
-        }
-        __nanosleep(64);
+    __threadfence();
+    const unsigned int old = atomicAdd(bar, blockIdx.x == 0 ? 0x80000000u - (gridDim.x - 1u) : 1u);
+    unsigned int polls = 0;
+    while ((((*reinterpret_cast<volatile unsigned int*>(bar)) ^ old) & 0x80000000u) == 0u) {
+      if (++polls > kOrthWaitPolls) {
+        gave_up = 1;
+        atomicExch(err, 1);
+        break;
       }
-      __threadfence();
+      __nanosleep(64);
     }
+    __threadfence();
   }
   __syncthreads();
-  if (gave_up) return;
-  scale_dot_dev(z, VB, hsub, n, partials, ticket, c_out, happy, VA2, c2_out, z32);
+  return !gave_up;
+}
+
+// ||z||_2 over a cooperative grid from the threads' sums of squares, known in
+// every CTA: behind one barrier each CTA adds up the partials itself (the same
+// sum in the same order as update_norm_dev's last CTA; one CTA summing and
+// publishing cost a second trip through L2).  CTA 0 publishes it.  rinv = 1 /
+// ||z||; false when nothing is to be scaled (breakdown, or the wait gave up).
+__device__ __forceinline__ bool inverse_norm_grid(double acc, double* partials, double* hsub, double tol, int* happy,
+                                                  int happy_value, unsigned int* bar, int* err, double& rinv) {
+  __shared__ double s_r;
+  __shared__ int s_go;
+  const double b = block_sum(acc);
+  if (threadIdx.x == 0) partials[blockIdx.x] = b;
+  if (!grid_barrier(bar, err)) return false;
+  const double sum = partials_sum(partials);
+  if (threadIdx.x == 0) {
+    const double r = sqrt(sum);
+    if (blockIdx.x == 0) norm_publish(r, hsub, tol, happy, happy_value);
+    s_go = !(r < tol);
+    s_r = 1.0 / r;
+  }
+  __syncthreads();
+  rinv = s_r;
+  return s_go != 0;
+}
+
+// Both passes in one launch of a grid whose CTAs are all resident at once (a
+// cooperative launch): the update, then, behind one barrier, the scaling of the
+// entries the threads still hold.  The same arithmetic in the same order as
+// update_norm_dev followed by scale_dev on the same grid (bitwise the same
+// results); it saves the second launch and its ramp, and z is read once and
+// written once.  Both passes, with the window's own products formed in the volume
+// kernel: 6 x 60 x 60, p = 5: 39.4 -> 30.6 us (the volume kernel 85 -> 90), 6 x 30
+// x 30: 23.4 -> 16.2 (29.5 -> 30.5), 6 x 4 x 4, p = 3: 14.4 -> 10.4.
+__device__ __forceinline__ void orth_fused_dev(double* __restrict__ z, const double* __restrict__ VA,
+                                               const double* __restrict__ VB, const double* h1p, const double* h2p,
+                                               long long n, double* partials, double* hsub, double tol, int* happy,
+                                               int happy_value, const double* __restrict__ VC, const double* h0p,
+                                               unsigned int* bar, int* err) {
+  // one round trip for the flag and the coefficients
+  const int broken = __ldcg(happy);
+  const double h1 = VA ? __ldcg(h1p) : 0.0, h2 = __ldcg(h2p), h0 = VC ? __ldcg(h0p) : 0.0;
+  if (broken) return;   // uniform over the grid
+  const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
+  double keep[kKeep];
+  const double acc = mgs_update_keep(z, VA, VB, h1, h2, i0, n, stride, VC, h0, keep);
+  double r;
+  if (inverse_norm_grid(acc, partials, hsub, tol, happy, happy_value, bar, err, r))
+    scale_keep(z, r, i0, n, stride, keep, nullptr);
 }
 
 // The window dots of the incomplete orthogonalisation as a pass of their own
@@ -461,14 +468,14 @@ __device__ __forceinline__ void orth_dots_range_t(const double* __restrict__ z, 
 // last forms the modified Gram-Schmidt coefficients from them exactly as the
 // volume epilogue does (h0 = z . V_{j-2}; h1 = z . V_{j-1} - h0 V_{j-1} . V_{j-2};
 // h2 = z . V_j - h0 V_j . V_{j-2} - h1 V_j . V_{j-1}, with the window's vectors
-// present) and stores V_j . V_{j-1}, V_j . V_{j-2} for the next iterations.
+// present) and stores V_j . V_{j-1} for the next iteration.
 // partials: 5 per CTA.  Returns 0 when the basis had already broken down
 // (nothing done), 2 in the CTA that finished last, else 1.
 __device__ __forceinline__ int orth_dots_dev(const double* __restrict__ z, const double* __restrict__ VB,
                                              const double* __restrict__ VA, const double* __restrict__ VC,
                                              long long n, double* partials, unsigned int* ticket, const int* happy,
                                              double* h0_out, double* h1_out, double* h2_out, double* cdot_out,
-                                             double* cdot2_out, const double* cprevAC) {
+                                             const double* cprevAC) {
   if (__ldcg(happy)) return 0;
   double s[5];
   const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
@@ -502,7 +509,6 @@ __device__ __forceinline__ int orth_dots_dev(const double* __restrict__ z, const
   if (threadIdx.x == 0) {
     const double a = u[0], bb = u[1], c3 = u[2];
     if (VA) *cdot_out = u[3];    // V_j . V_{j-1}
-    if (VC) *cdot2_out = u[4];   // V_j . V_{j-2}
     if (VC) {
       const double h0 = c3;
       const double h1 = a - h0 * __ldcg(cprevAC);
@@ -550,25 +556,24 @@ __device__ __forceinline__ bool grid_step(unsigned int* gen, unsigned int target
 
 // The dot pass, the update pass and the scale pass of the complex64-bulk form
 // in one cooperative launch (two grid-wide steps); the same arithmetic in the
-// same order as orth_dots_dev, update_norm_dev and scale_dot_dev on the same
+// same order as orth_dots_dev, update_norm_dev and scale_dev on the same
 // grid.  The H entries and the norm pass between the phases through L2.
 __device__ __forceinline__ void orth3_fused_dev(double* __restrict__ z, const double* __restrict__ VA,
                                                 const double* __restrict__ VB, const double* __restrict__ VC,
                                                 long long n, double* partials, unsigned int* ticket, double tol,
                                                 int* happy, int happy_value, double* h0p, double* h1p, double* h2p,
-                                                double* hsub, double* cdot_out, double* cdot2_out,
-                                                const double* cprevAC, float* __restrict__ z32, unsigned int* gen,
+                                                double* hsub, double* cdot_out, const double* cprevAC, float* __restrict__ z32, unsigned int* gen,
                                                 int* err) {
   __shared__ unsigned int g0;
   // read before this CTA's first ticket (ordered by the fence ahead of it)
   if (threadIdx.x == 0) g0 = *reinterpret_cast<volatile unsigned int*>(gen);
-  int st = orth_dots_dev(z, VB, VA, VC, n, partials, ticket, happy, h0p, h1p, h2p, cdot_out, cdot2_out, cprevAC);
+  int st = orth_dots_dev(z, VB, VA, VC, n, partials, ticket, happy, h0p, h1p, h2p, cdot_out, cprevAC);
   if (st == 0) return;   // uniform over the grid
   if (!grid_step(gen, g0 + 1u, st == 2, err)) return;
   st = update_norm_dev(z, VA, VB, h1p, h2p, n, partials, ticket, hsub, tol, happy, happy_value, VC, h0p);
   if (st == 0) return;
   if (!grid_step(gen, g0 + 2u, st == 2, err)) return;
-  scale_dot_dev(z, VB, hsub, n, partials, ticket, nullptr, happy, nullptr, nullptr, z32);
+  scale_dev(z, hsub, n, happy, z32);
 }
 
 // ------------------------------------------------------------ expm

@@ -114,7 +114,6 @@ struct Ctx {
   double* d_partials = nullptr;   // reduction partials
   double* d_vpart = nullptr;      // partials of the epilogue dot products (2 per volume block)
   double* d_cdot = nullptr;       // V_j . V_{j-1} per basis index
-  double* d_cdot2 = nullptr;      // V_j . V_{j-2} per basis index (window of three)
   double* d_scal = nullptr;       // device scalars (see kiops.cu)
   int* d_flags = nullptr;         // happy flag, happy size
   double* h_pinned = nullptr;     // pinned read-back area
@@ -247,25 +246,18 @@ struct AugEpilogue {
   // incomplete orthogonalisation fused into the epilogue (window of two or
   // three): with dotB set, the modified Gram-Schmidt coefficients of z against
   // V_C = V_{j-2}, V_A = V_{j-1}, V_B = V_j (oldest first) are formed from the
-  // dots z . V over the augmented length n + p and the stored V . V products:
+  // dots z . V and V . V over the augmented length n + p:
   //   h0 = V_C . z,  h1 = V_A . z - h0 (V_A . V_C),
   //   h2 = V_B . z - h0 (V_B . V_C) - h1 (V_B . V_A)
   // (block partials, last block finalises); absent vectors drop their terms
   const double* dotA = nullptr;     // V_{j-1} (null for the first basis vector)
   const double* dotB = nullptr;     // V_j
   const double* dotC = nullptr;     // V_{j-2} (window of three, j >= 2)
-  const double* cprev = nullptr;    // V_j . V_{j-1}
-  const double* cprevC = nullptr;   // V_j . V_{j-2}
-  const double* cprevAC = nullptr;  // V_{j-1} . V_{j-2}
+  const double* cprevAC = nullptr;  // V_{j-1} . V_{j-2} (the previous iteration's cdot_out)
+  double* cdot_out = nullptr;       // receives V_j . V_{j-1} (with dotA)
   double* h0_out = nullptr;
   double* h1_out = nullptr;
   double* h2_out = nullptr;
-  // with cdot_out set, V_j . V_{j-1} (and, window of three, V_j . V_{j-2}) are
-  // formed here from the window vectors and written there, instead of being
-  // read from cprev / cprevC (complex64-bulk form: the scale pass then forms
-  // no dots)
-  double* cdot_out = nullptr;
-  double* cdot2_out = nullptr;
   double* dpart = nullptr;          // 5 doubles per block
   unsigned int* dticket = nullptr;
   long long n = 0;
@@ -289,14 +281,20 @@ int launch_jvp_fb(Ctx& c, const double* q, const double* v, double eps, double* 
 
 // ---- Krylov kernels (krylov.cu)
 constexpr int RED_BLOCKS = 608;   // 4 x 152 SMs
-// CTAs of a reduction or vector pass over n entries (256 threads each): two
-// entries a thread until the GPU is full.  Every CTA takes a ticket, and in the
-// cooperative pass waits for the last one, so idle CTAs cost time: at n = 4608
-// (6 x 4 x 4, p = 3) the two passes take 14.4 us with ten CTAs, 18.4 with 608.
-inline int red_blocks(long long n) {
+// CTAs of a reduction over n entries (256 threads each): two entries a thread
+// until the GPU is full; every CTA takes a ticket, so idle ones cost time
+inline int capped_blocks(long long n, int cap) {
   const long long b = (n + 511) / 512;
-  return (int)(b < 1 ? 1 : (b > RED_BLOCKS ? RED_BLOCKS : b));
+  return (int)(b < 1 ? 1 : (b > cap ? cap : b));
 }
+inline int red_blocks(long long n) { return capped_blocks(n, RED_BLOCKS); }
+// CTAs of the FP64 path's orthogonalisation passes (krylov_device.cuh): two per
+// SM, so that a thread has the registers to keep its entries of z from phase to
+// phase.  The complex64-bulk form's three phases take RED_BLOCKS: with 304 and z
+// kept they were no faster (68 against 66 us at 6 x 60 x 60, p = 5; the five
+// dots, not the traffic of z, bound them) and the step lost 8 us around them.
+constexpr int ORTH_BLOCKS = 304;
+inline int orth_blocks(long long n) { return capped_blocks(n, ORTH_BLOCKS); }
 int launch_dot(Ctx& c, const double* x, const double* y, long long n, double* dst, const int* skip,
                cudaStream_t s);
 int launch_norm2(Ctx& c, const double* x, long long n, double* dst, double tol, int* happy,
@@ -315,34 +313,33 @@ int launch_combine(Ctx& c, int j, long long n, cudaStream_t s);
 int launch_to_float_scaled(Ctx& c, const double* src, float* dst, long long n, double scale, cudaStream_t s);
 // fused incomplete orthogonalisation (window two or three) after an epilogue
 // with dots: z -= h0 V_C + h1 V_A + h2 V_B and ||z|| -> *hsub (happy flag below
-// tol), then V_next = z / *hsub, V_next . V_B -> *c_out and, with V_A given,
-// V_next . V_A -> *c2_out
+// tol), then V_next = z / *hsub (with z32 also its FP32 copy)
 int launch_update_norm(Ctx& c, double* z, const double* VA, const double* VB, const double* h1, const double* h2,
-                       long long N, double* hsub, double tol, int happy_value, cudaStream_t s,
+                       long long N, double* hsub, double tol, int happy_value, int blocks, cudaStream_t s,
                        const double* VC = nullptr, const double* h0 = nullptr);
-int launch_scale_dot(Ctx& c, double* z, const double* VB, const double* hsub, long long N, double* c_out,
-                     cudaStream_t s, const double* VA = nullptr, double* c2_out = nullptr, float* z32 = nullptr);
+int launch_scale(Ctx& c, double* z, const double* hsub, long long N, int blocks, cudaStream_t s,
+                 float* z32 = nullptr);
 // dst = src rounded to FP32 (n entries)
 int launch_to_float(Ctx& c, const double* src, float* dst, long long n, cudaStream_t s);
-// both orthogonalisation passes (launch_update_norm, then launch_scale_dot with
-// c_out, VA2, c2_out, z32) in one cooperative launch, where the GPU holds its
-// whole grid at once (orth_fused_available); a wait past its bound sets d_flags[3]
+// both orthogonalisation passes (launch_update_norm, then launch_scale) in one
+// cooperative launch, where the GPU holds its whole grid at once
+// (orth_fused_available); a wait past its bound sets d_flags[3]
 int orth_fused_available(Ctx& c);
-// the complex64-bulk form's window dots as a pass of their own (its FP32
-// volume kernel forms none): the five sums over the augmented vectors, the
-// modified Gram-Schmidt coefficients into the H entries, V_j . V_{j-1} and
-// V_j . V_{j-2} into cdot_out, cdot2_out (orth_dots_dev)
-int launch_orth_dots(Ctx& c, const double* z, const double* VB, const double* VA, const double* VC, long long N,
-                     double* h0_out, double* h1_out, double* h2_out, double* cdot_out, double* cdot2_out,
-                     const double* cprevAC, cudaStream_t s);
-// that pass, the update pass and the scale pass (no dots, the FP32 copy z32)
-// in one cooperative launch, where orth_fused_available
-int launch_orth3_fused(Ctx& c, double* z, const double* VA, const double* VB, const double* VC, long long N,
-                       double tol, int happy_value, double* h0p, double* h1p, double* h2p, double* hsub,
-                       double* cdot_out, double* cdot2_out, const double* cprevAC, float* z32, cudaStream_t s);
 int launch_orth_fused(Ctx& c, double* z, const double* VA, const double* VB, const double* h1, const double* h2,
                       long long N, double* hsub, double tol, int happy_value, const double* VC, const double* h0,
-                      double* c_out, const double* VA2, double* c2_out, float* z32, cudaStream_t s);
+                      cudaStream_t s);
+// the complex64-bulk form's window dots as a pass of their own (its FP32
+// volume kernel forms none): the five sums over the augmented vectors, the
+// modified Gram-Schmidt coefficients into the H entries, V_j . V_{j-1} into
+// cdot_out (orth_dots_dev)
+int launch_orth_dots(Ctx& c, const double* z, const double* VB, const double* VA, const double* VC, long long N,
+                     double* h0_out, double* h1_out, double* h2_out, double* cdot_out, const double* cprevAC,
+                     cudaStream_t s);
+// that pass, the update pass and the scale pass (with the FP32 copy z32) in one
+// cooperative launch, where orth_fused_available
+int launch_orth3_fused(Ctx& c, double* z, const double* VA, const double* VB, const double* VC, long long N,
+                       double tol, int happy_value, double* h0p, double* h1p, double* h2p, double* hsub,
+                       double* cdot_out, const double* cprevAC, float* z32, cudaStream_t s);
 double fp64_fma_peak_tflops();
 int launch_set_tail(Ctx& c, double* x, long long n, int p, const double* vals, cudaStream_t s);
 int launch_lincomb(Ctx& c, double* out, long long n, int k, const double* const* xs,
