@@ -308,6 +308,7 @@ void sw_free(sw_ctx_t c) {
                     c->d_partials, c->d_scal, c->d_Fn, c->d_tmp, c->d_tmp2, c->d_lin_node, c->d_lin_face,
                     c->d_vpart, c->d_cdot, c->d_diag_tab, c->d_diag_part, c->d_diag_out, c->d_qhost};
   if (c->d_diag_flags) cudaFree(c->d_diag_flags);
+  if (c->d_lin_exp) cudaFree(c->d_lin_exp);
   if (c->d_lin_node32) cudaFree(c->d_lin_node32);
   if (c->d_lin_face32) cudaFree(c->d_lin_face32);
   if (c->d_b32) cudaFree(c->d_b32);

@@ -160,7 +160,8 @@ __global__ void __launch_bounds__(VolShape<NS>::THREADS) volume_kernel(VolArgs a
   // DFR sweeps: extended flux [F(-1), f_1..f_NS, F(+1)] per line (Eq. 11-14)
   double res[3] = {0.0, 0.0, 0.0};
   if (active) {
-    fx_sweep<NS>(sm.sF[le], &sm.sB[le][0][0][0], k1, k2, sm.sD[k1], sm.sD[k2], dc, dscale, fixed, m0, m1, S1, S2, res);
+    fx_sweep<NS, true>(sm.sF[le], &sm.sB[le][0][0][0], k1, k2, sm.sD[k1], sm.sD[k2], dc, dscale, fixed, fx_exp(m0),
+                       fx_exp(m1), 0, 0, S1, S2, res);
     if (a.v) {
       const double sc = 1.0 / a.eps;
 #pragma unroll

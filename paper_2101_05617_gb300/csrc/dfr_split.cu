@@ -10,7 +10,7 @@
 // point, the coefficients of the imaginary half:
 //   lin_node_kernel   per node: u^1, u^2 and the coefficients of the imaginary
 //                     parts of sqrt(g) T^{ij} (Eq. 136) and of the sources of
-//                     Eq. (2) as functions of Im q;
+//                     Eq. (2) as functions of Im q, packed for block fixed point;
 //   lin_face_kernel   per interface point: the 3 x 6 matrix taking the
 //                     imaginary parts of the two traces to the imaginary part of
 //                     the AUSM flux: what propagating unit imaginary parts
@@ -19,9 +19,9 @@
 //                     transform folded in).
 // Each JVP then runs only the imaginary half, in real arithmetic:
 //   face_tangent_kernel   traces of v, the 3 x 6 map, the hand-back;
-//   volume_tangent_kernel pointwise imaginary fluxes and sources, the DFR
-//                         sweeps (Eq. 12-14; in FP64 as block fixed point on the
-//                         integer pipe, fixed.cuh) and the augmented-operator
+//   volume_tangent_kernel pointwise imaginary fluxes and sources and the DFR
+//                         sweeps (Eq. 12-14; in FP64 both as block fixed point on
+//                         the integer pipe, fixed.cuh), and the augmented-operator
 //                         epilogue.
 // The imaginary parts are proportional to eps, so the tangent is propagated for
 // v itself and the final division by eps is omitted.  Results equal the plain
@@ -40,30 +40,79 @@ namespace swepi {
 namespace {
 
 // ---------------------------------------------------------------- linearise
-__global__ void lin_node_kernel(const double* __restrict__ q, const double* __restrict__ nc, long long nodes,
-                                double* __restrict__ ln) {
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nodes) return;
-  const long long N = nodes;
-  const double q0 = q[i], q1 = q[i + N], q2 = q[i + 2 * N];
-  const double r = 1.0 / q0;
-  const double u1 = q1 * r, u2 = q2 * r;
-  const double c11 = nc[NC_C11 * N + i], c12 = nc[NC_C12 * N + i], c22 = nc[NC_C22 * N + i];
-  const double g1a = nc[NC_G1A * N + i], g1b = nc[NC_G1B * N + i];
-  const double g2a = nc[NC_G2A * N + i], g2b = nc[NC_G2B * N + i];
-  // Im sqrt(g)T^{ij} = u^j Im q^i + u^i Im q^j + (g_r h^ij q^0 / sqrt g - u^i u^j) Im q^0
-  ln[LN_U1 * N + i] = u1;
-  ln[LN_U2 * N + i] = u2;
-  ln[LN_A11 * N + i] = 2.0 * c11 * q0 - u1 * u1;
-  ln[LN_A12 * N + i] = 2.0 * c12 * q0 - u1 * u2;
-  ln[LN_A22 * N + i] = 2.0 * c22 * q0 - u2 * u2;
-  // Im S^i = s_i1 Im q^1 + s_i2 Im q^2 + s_i0 Im q^0 (Coriolis, Gamma^i_jk, topography terms of Eq. 2)
-  ln[LN_S11 * N + i] = nc[NC_K11 * N + i] - 2.0 * g1a * u1 - g1b * u2;
-  ln[LN_S12 * N + i] = nc[NC_K12 * N + i] - g1b * u1;
-  ln[LN_S10 * N + i] = g1a * u1 * u1 + g1b * u1 * u2 + nc[NC_B1 * N + i];
-  ln[LN_S21 * N + i] = nc[NC_K21 * N + i] - g2a * u2;
-  ln[LN_S22 * N + i] = nc[NC_K22 * N + i] - g2a * u1 - 2.0 * g2b * u2;
-  ln[LN_S20 * N + i] = g2a * u1 * u2 + g2b * u2 * u2 + nc[NC_B2 * N + i];
+// The coefficients are packed for the block fixed-point products (fixed.cuh,
+// dfr_tangent.cuh) with the exponents per element that their sums need: u for
+// the u^i, a for the A^{ij}, s for the S^i_j, s0 for the S^i_0, with
+//   s0 - s = a - u       (the terms of a source come out in one unit) and
+//   k = De + u - s >= 0  (a source adds to the packed sweep after a right shift).
+// The sources are stored times -dx/2: the sweep's sums and they share the factor
+// -2/dx.  An element with a coefficient past the format's range keeps FP64 values.
+// ln32 (complex64-bulk form): the unscaled coefficients rounded to FP32.
+template <int NS>
+__global__ void __launch_bounds__(VolShape<NS>::THREADS) lin_node_kernel(const double* __restrict__ q,
+                                                                         const double* __restrict__ nc, long long nodes,
+                                                                         double mhdx, int De, double* __restrict__ ln,
+                                                                         int4* __restrict__ le,
+                                                                         float* __restrict__ ln32) {
+  constexpr int NN = NS * NS, EPB = VolShape<NS>::EPB, THREADS = VolShape<NS>::THREADS;
+  __shared__ unsigned sE[2][EPB][2];
+  for (int t = threadIdx.x; t < 4 * EPB; t += THREADS) (&sE[0][0][0])[t] = 0u;
+  const long long i = (long long)blockIdx.x * THREADS + threadIdx.x, N = nodes;
+  const int e = threadIdx.x / NN;
+  const bool active = i < nodes;
+  double c[LN_COUNT];
+  unsigned mu = 0u, ma = 0u, ms = 0u, ms0 = 0u;
+  if (active) {
+    const double q0 = q[i], q1 = q[i + N], q2 = q[i + 2 * N];
+    const double r = 1.0 / q0;
+    const double u1 = q1 * r, u2 = q2 * r;
+    const double c11 = nc[NC_C11 * N + i], c12 = nc[NC_C12 * N + i], c22 = nc[NC_C22 * N + i];
+    const double g1a = nc[NC_G1A * N + i], g1b = nc[NC_G1B * N + i];
+    const double g2a = nc[NC_G2A * N + i], g2b = nc[NC_G2B * N + i];
+    // Im sqrt(g)T^{ij} = u^j Im q^i + u^i Im q^j + (g_r h^ij q^0 / sqrt g - u^i u^j) Im q^0
+    c[LN_U1] = u1;
+    c[LN_U2] = u2;
+    c[LN_A11] = 2.0 * c11 * q0 - u1 * u1;
+    c[LN_A12] = 2.0 * c12 * q0 - u1 * u2;
+    c[LN_A22] = 2.0 * c22 * q0 - u2 * u2;
+    // Im S^i = s_i1 Im q^1 + s_i2 Im q^2 + s_i0 Im q^0 (Coriolis, Gamma^i_jk, topography terms of Eq. 2)
+    c[LN_S11] = nc[NC_K11 * N + i] - 2.0 * g1a * u1 - g1b * u2;
+    c[LN_S12] = nc[NC_K12 * N + i] - g1b * u1;
+    c[LN_S10] = g1a * u1 * u1 + g1b * u1 * u2 + nc[NC_B1 * N + i];
+    c[LN_S21] = nc[NC_K21 * N + i] - g2a * u2;
+    c[LN_S22] = nc[NC_K22 * N + i] - g2a * u1 - 2.0 * g2b * u2;
+    c[LN_S20] = g2a * u1 * u2 + g2b * u2 * u2 + nc[NC_B2 * N + i];
+    if (ln32) {
+#pragma unroll
+      for (int k = 0; k < LN_COUNT; ++k) ln32[k * N + i] = (float)c[k];
+    }
+#pragma unroll
+    for (int k = LN_S11; k < LN_COUNT; ++k) c[k] *= mhdx;
+    mu = max(fx_key(c[LN_U1]), fx_key(c[LN_U2]));
+    ma = max(fx_key(c[LN_A11]), max(fx_key(c[LN_A12]), fx_key(c[LN_A22])));
+    ms = max(max(fx_key(c[LN_S11]), fx_key(c[LN_S12])), max(fx_key(c[LN_S21]), fx_key(c[LN_S22])));
+    ms0 = max(fx_key(c[LN_S10]), fx_key(c[LN_S20]));
+  }
+  __syncthreads();
+  fx_block_max<NN, EPB, THREADS>(sE[0], e, mu, ma);
+  fx_block_max<NN, EPB, THREADS>(sE[1], e, ms, ms0);
+  __syncthreads();
+  if (!active) return;
+  mu = sE[0][e][0];
+  ma = sE[0][e][1];
+  ms = sE[1][e][0];
+  ms0 = sE[1][e][1];
+  const bool packed = fx_usable(mu) && fx_usable(ma) && fx_usable(ms) && fx_usable(ms0);
+  // an all-zero class takes the smallest exponent and constrains nothing
+  const int eu = mu ? (int)(mu >> 20) : kFxExpMin, ea = ma ? (int)(ma >> 20) : kFxExpMin;
+  const int es = ms ? (int)(ms >> 20) : kFxExpMin, es0 = ms0 ? (int)(ms0 >> 20) : kFxExpMin;
+  const int u = max(eu, es - De), a = max(ea, es0 - es + u), s0 = es + a - u;
+  if (threadIdx.x % NN == 0) le[i / NN] = packed ? make_int4(u, a, De + u - es, 1) : make_int4(0, 0, 0, 0);
+#pragma unroll
+  for (int k = 0; k < LN_COUNT; ++k) {
+    const int E = k <= LN_U2 ? u : (k <= LN_A22 ? a : ((k == LN_S10 || k == LN_S20) ? s0 : es));
+    ln[k * N + i] = packed ? fx_pack(c[k], E) : c[k];
+  }
 }
 
 struct LinFaceArgs {
@@ -200,8 +249,10 @@ __global__ void to_float_kernel(const double* __restrict__ src, float* __restric
 
 template <int NS>
 int linearize_ns(Ctx& c, const double* q, cudaStream_t s) {
-  const int th = 256;
-  lin_node_kernel<<<(unsigned)((c.nodes + th - 1) / th), th, 0, s>>>(q, c.d_node_coef, c.nodes, c.d_lin_node);
+  const int th = VolShape<NS>::THREADS;
+  lin_node_kernel<NS><<<(unsigned)((c.nodes + th - 1) / th), th, 0, s>>>(
+      q, c.d_node_coef, c.nodes, -0.5 * c.dx, c.dc.dq_exp + 1080, c.d_lin_node, c.d_lin_exp,
+      c.jvp_mode == 2 ? c.d_lin_node32 : nullptr);
   LinFaceArgs fa{q, c.nodes, c.d_lines, c.d_face_coef, c.nfacepts, c.d_lin_face};
   lin_face_kernel<NS><<<(unsigned)((c.nfacepts + 127) / 128), 128, 0, s>>>(fa, c.dc);
   c.launches += 2;
@@ -226,7 +277,7 @@ int tangent_ns(Ctx& c, const double* v, double* out, const AugEpilogue& ep, cons
     e1 = prof_event(c);
     cudaEventRecord(e1, s);
   }
-  TanVolArgs<T> va{v, c.nodes, c.nelem, ln, fb, out, ep};
+  TanVolArgs<T> va{v, c.nodes, c.nelem, ln, c.d_lin_exp, fb, out, ep};
   const long long vblocks = (c.nelem + VolShape<NS>::EPB - 1) / VolShape<NS>::EPB;
   int rt = 1;
   if (sizeof(T) == 4) {   // complex64-bulk form: element tiles staged by bulk copies where aligned
@@ -275,7 +326,7 @@ int capture_iter_ns(Ctx& c, KDev* kd, const KFix& f, bool w3, int p, cudaStream_
     const int rt = capture_volume_tile_dev<NS>(c, kd, f, w3, s);
     if (rt <= 0) return rt;
   }
-  TanVolArgs<T> va{nullptr, c.nodes, c.nelem, ln, fb, nullptr, AugEpilogue{}};
+  TanVolArgs<T> va{nullptr, c.nodes, c.nelem, ln, c.d_lin_exp, fb, nullptr, AugEpilogue{}};
   const long long vblocks = (c.nelem + VolShape<NS>::EPB - 1) / VolShape<NS>::EPB;
   const int ctas = w3 ? volume_ctas<T, NS, true, true>(c.device, vblocks)
                       : volume_ctas<T, NS, false, true>(c.device, vblocks);
@@ -333,6 +384,15 @@ int capture_iter_jvp(Ctx& c, KDev* kd, const KFix& f, bool fp32, bool w3, int p,
 int launch_linearize(Ctx& c, const double* q, cudaStream_t s) {
   if (!c.d_lin_node && cudaMalloc(&c.d_lin_node, sizeof(double) * LN_COUNT * c.nodes) != cudaSuccess)
     return SW_ENOMEM;
+  if (!c.d_lin_exp && cudaMalloc(&c.d_lin_exp, sizeof(int4) * c.nelem) != cudaSuccess) return SW_ENOMEM;
+  if (c.jvp_mode == 2) {
+    // complex64-bulk form: FP32 copies of the coefficient tables
+    if (!c.d_lin_node32 && cudaMalloc(&c.d_lin_node32, sizeof(float) * LN_COUNT * c.nodes) != cudaSuccess)
+      return SW_ENOMEM;
+    if (!c.d_lin_face32 && cudaMalloc(&c.d_lin_face32, sizeof(float) * 23 * c.nfacepts) != cudaSuccess)
+      return SW_ENOMEM;
+    if (!c.d_v32 && cudaMalloc(&c.d_v32, sizeof(float) * c.n) != cudaSuccess) return SW_ENOMEM;
+  }
   if (!c.d_lin_face && cudaMalloc(&c.d_lin_face, sizeof(double) * 18 * c.nfacepts) != cudaSuccess)
     return SW_ENOMEM;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -355,18 +415,11 @@ int launch_linearize(Ctx& c, const double* q, cudaStream_t s) {
     default: return SW_EINVAL;
   }
   if (rc == SW_OK && c.jvp_mode == 2) {
-    // complex64-bulk form: FP32 copies of the coefficient tables
-    if (!c.d_lin_node32 && cudaMalloc(&c.d_lin_node32, sizeof(float) * LN_COUNT * c.nodes) != cudaSuccess)
-      return SW_ENOMEM;
-    if (!c.d_lin_face32 && cudaMalloc(&c.d_lin_face32, sizeof(float) * 23 * c.nfacepts) != cudaSuccess)
-      return SW_ENOMEM;
-    if (!c.d_v32 && cudaMalloc(&c.d_v32, sizeof(float) * c.n) != cudaSuccess) return SW_ENOMEM;
-    to_float_kernel<<<1024, 256, 0, s>>>(c.d_lin_node, c.d_lin_node32, (long long)LN_COUNT * c.nodes);
     to_float_kernel<<<1024, 256, 0, s>>>(c.d_lin_face, c.d_lin_face32, 18LL * c.nfacepts);
     // M00, M01, M10, M11, sigma (consecutive rows of the face table) after the map rows
     to_float_kernel<<<1024, 256, 0, s>>>(c.d_face_coef + (long long)FC_M00 * c.nfacepts,
                                          c.d_lin_face32 + 18LL * c.nfacepts, 5LL * c.nfacepts);
-    c.launches += 3;
+    c.launches += 2;
     rc = cuda_status(cudaGetLastError());
   }
   if (pl) {

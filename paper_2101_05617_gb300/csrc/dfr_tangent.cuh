@@ -117,6 +117,7 @@ struct TanVolArgs {
   long long nodes;
   long long nelem;
   const T* ln;
+  const int4* le;   // FP64: exponents of the packed coefficients per element
   const T* fb;
   double* out;
   AugEpilogue ep;
@@ -187,10 +188,9 @@ __device__ __forceinline__ void tile_fluxes(const TanVolArgs<T>& a, VolSmem<T, N
 // the sweeps run as integer multiply-adds.  An element that the format cannot
 // hold keeps FP64 values in the same arrays and takes the FP64 chain.
 // 6 x 60 x 60, p = 5, with the augmented operator and the window dots: 134 ->
-// 85 us (FP64 pipe 87 -> 66 %: ~41 FP64 instructions a node are left of 83, the
-// point fluxes 15, the b columns 12, the window dots 6); the product alone 129
-// -> 79 us with its face kernel, 6 x 90 x 90, p = 6: 395 -> 217 us.  Relative
-// error against a 64-bit reference unchanged (3.5e-15, the reference's own).
+// 85 us (FP64 pipe 87 -> 66 %); the product alone 129 -> 79 us with its face
+// kernel, 6 x 90 x 90, p = 6: 395 -> 217 us.  Relative error against a 64-bit
+// reference unchanged (3.5e-15, the reference's own).
 
 // what one node brings to its element: its fluxes, and its share of the
 // element's 12 N_s interface fluxes
@@ -256,16 +256,18 @@ __device__ __forceinline__ bool fx_scale_usable(double s) {
 }
 
 // the two sweeps of node (k2, k1): res[mu] = dscale * (D-row k1 along xi^1 +
-// D-row k2 along xi^2) + add[mu] (add[0] is zero).  Da, Db: the packed rows in
+// D-row k2 along xi^2 + isrc[mu]) + add[mu] for mu = 1, 2 (isrc in units of the
+// packed sums, where `fixed`).  E0, E1: the block exponents.  ADD:
+// whether add1, add2 are added where `fixed`.  Da, Db: the packed rows in
 // shared memory (each entry read once for the three variables: rows held in
 // registers spilled); sB [4][3][NS].  The packed sum is converted once (one
 // FP64 instruction) and scaled by dscale with the blocks' exponents added to
 // its exponent field.
-template <int NS>
+template <int NS, bool ADD>
 __device__ __forceinline__ void fx_sweep(const double (*sF)[3][NS * NS], const double* sB, int k1, int k2,
                                          const double* Da, const double* Db, const DfrConst& dc,
-                                         double dscale, bool fixed, unsigned M0, unsigned M1, double add1, double add2,
-                                         double res[3]) {
+                                         double dscale, bool fixed, int E0, int E1, long long isrc1, long long isrc2,
+                                         double add1, double add2, double res[3]) {
   if (fixed) {
     FxAcc a[3];
 #pragma unroll
@@ -285,10 +287,13 @@ __device__ __forceinline__ void fx_sweep(const double (*sF)[3][NS * NS], const d
     const int sh = __double2hiint(dscale), sl = __double2loint(dscale);
 #pragma unroll
     for (int mu = 0; mu < 3; ++mu) {
-      const int k = fx_exp(mu == 0 ? M0 : M1) + dc.dq_exp;
+      const int k = (mu == 0 ? E0 : E1) + dc.dq_exp;
       const double sc = __hiloint2double(sh + k * 1048576, sl);
+      if (mu == 1) a[mu].hh += isrc1;
+      if (mu == 2) a[mu].hh += isrc2;
       const double s = fx_sum(a[mu]);
-      res[mu] = mu == 0 ? s * sc : fma(s, sc, mu == 1 ? add1 : add2);
+      if constexpr (ADD) res[mu] = mu == 0 ? s * sc : fma(s, sc, mu == 1 ? add1 : add2);
+      else res[mu] = s * sc;
     }
     return;
   }
@@ -309,21 +314,150 @@ __device__ __forceinline__ void fx_sweep(const double (*sF)[3][NS * NS], const d
   }
 }
 
-// pointwise imaginary fluxes of node idx into pt, the sources S^1, S^2 returned
+// ---- FP64: the point fluxes in block fixed point too
+// Im sqrt(g) T^{ij} and Im S^i are sums of coefficient times v.  The
+// coefficients are packed once per linearisation point (lin_node_kernel), with
+// exponents per element for four classes: u for u^i, a for the A^{ij}, s for the
+// S^i_j and s0 = s + a - u for the S^i_0, so that packing v^1, v^2 for the
+// exponent EU = t + 2 - u and v^0 for EA = t + 2 - a puts all terms in one unit and
+// the fluxes come out as block values of exponent TF = t - 1020, t the largest of
+// a + e(v^0), u + e(v^i) and e(interface flux) + 1020 in the element (e: biased
+// exponents; the two spare bits are the sums' headroom).  The sources, stored
+// times -dx/2, add to the packed sweep shifted by k = De + u - s >= 0.  What is
+// left for the FP64 pipe is the conversion and scaling of three sums a node.
+// 6 x 60 x 60, p = 5: 90 -> 81 us with the augmented operator and the dots, the
+// product with its face kernel 71 -> 67 us; 6 x 90 x 90, p = 6: 217 -> 188 us.
+struct LinExp {
+  int u, a, k, packed;
+};
+__device__ __forceinline__ LinExp lin_exp(const int4* __restrict__ le, long long elem) {
+  const int4 x = __ldg(le + elem);
+  return {x.x, x.y, x.z, x.w};
+}
+// a value's bid for t: its exponent plus off; zeros (and subnormals) none, and
+// one past the format's range a bid past every limit
+__device__ __forceinline__ unsigned fx_bid(double x, int off) {
+  const int e = (__double2hiint(x) >> 20) & 0x7ff;
+  return e == 0 ? 0u : (e > kFxExpMax ? 1u << 14 : (unsigned)(e + off));
+}
+__device__ __forceinline__ bool fx_bid_usable(unsigned t) {
+  return t == 0u || (t >= 1020u + kFxExpMin && t <= 1020u + kFxExpMax);
+}
+
+// what one node brings to its element before the exponents are known
 template <int NS>
-__device__ __forceinline__ void tan_fluxes(const TanVolArgs<double>& a, long long idx, FxPoint<NS>& pt, double& S1,
-                                           double& S2) {
+struct TanPoint {
+  static constexpr int EC = (12 + NS - 1) / NS;   // interface values per thread
+  double v0, v1, v2;
+  double e[EC];
+};
+template <int NS>
+__device__ __forceinline__ void tan_load(const TanVolArgs<double>& a, long long elem, int node, long long idx,
+                                         const LinExp& x, TanPoint<NS>& pt, unsigned& m0, unsigned& t) {
+  constexpr int NN = NS * NS;
   const long long N = a.nodes;
-  const double v0 = __ldg(a.v + idx), v1 = __ldg(a.v + idx + N), v2 = __ldg(a.v + idx + 2 * N);
+  pt.v0 = __ldg(a.v + idx);
+  pt.v1 = __ldg(a.v + idx + N);
+  pt.v2 = __ldg(a.v + idx + 2 * N);
+#pragma unroll
+  for (int i = 0; i < TanPoint<NS>::EC; ++i) {
+    const int r = node + i * NN;
+    pt.e[i] = 0.0;
+    if (r < 12 * NS) {
+      pt.e[i] = a.fb[elem * 12 * NS + r];
+      if ((r / NS) % 3 == 0) m0 = max(m0, fx_key(pt.e[i]));
+      else t = max(t, fx_bid(pt.e[i], 1020));
+    }
+  }
+  m0 = max(m0, max(fx_key(pt.v1), fx_key(pt.v2)));
+  t = max(t, max(fx_bid(pt.v0, x.a), max(fx_bid(pt.v1, x.u), fx_bid(pt.v2, x.u))));
+}
+
+// the node's fluxes and interface values into the tile's arrays of its element,
+// and its sources (times -dx/2): where `fixed` packed, s1 and s2 in units of the
+// sweep's sums; else FP64, s1 and s2 holding their bits
+template <int NS>
+__device__ __forceinline__ void tan_fluxes(const TanVolArgs<double>& a, double (*sF)[3][NS * NS], double* sB, int node,
+                                           long long idx, const LinExp& x, const TanPoint<NS>& pt, int De,
+                                           bool fixed, unsigned M0, unsigned t, long long& s1, long long& s2) {
+  constexpr int NN = NS * NS;
+  const long long N = a.nodes;
   const double* ln = a.ln + idx;
-  const double u1 = ln[LN_U1 * N], u2 = ln[LN_U2 * N];
-  pt.F11 = fma(2.0 * u1, v1, ln[LN_A11 * N] * v0);
-  pt.F12 = fma(u2, v1, fma(u1, v2, ln[LN_A12 * N] * v0));
-  pt.F22 = fma(2.0 * u2, v2, ln[LN_A22 * N] * v0);
-  S1 = fma(ln[LN_S11 * N], v1, fma(ln[LN_S12 * N], v2, ln[LN_S10 * N] * v0));
-  S2 = fma(ln[LN_S21 * N], v1, fma(ln[LN_S22 * N], v2, ln[LN_S20 * N] * v0));
-  pt.v1 = v1;
-  pt.v2 = v2;
+  if (fixed) {
+    const int E0 = fx_exp(M0), TF = t == 0u ? 1023 : (int)t - 1020;
+    const double p0 = fx_pack(pt.v0, TF + 1022 - x.a);
+    const double p1 = fx_pack(pt.v1, TF + 1022 - x.u), p2 = fx_pack(pt.v2, TF + 1022 - x.u);
+    sF[0][0][node] = fx_pack(pt.v1, E0);
+    sF[1][0][node] = fx_pack(pt.v2, E0);
+    const double u1 = ln[LN_U1 * N], u2 = ln[LN_U2 * N];
+    FxAcc f;
+    fx_mac(f, u1, p1);
+    f.hh += f.hh;
+    f.mid += f.mid;
+    fx_mac(f, ln[LN_A11 * N], p0);
+    sF[0][1][node] = fx_repack(fx_int(f));
+    f = FxAcc();
+    fx_mac(f, u2, p1);
+    fx_mac(f, u1, p2);
+    fx_mac(f, ln[LN_A12 * N], p0);
+    const double f12 = fx_repack(fx_int(f));
+    sF[0][2][node] = f12;
+    sF[1][1][node] = f12;
+    f = FxAcc();
+    fx_mac(f, u2, p2);
+    f.hh += f.hh;
+    f.mid += f.mid;
+    fx_mac(f, ln[LN_A22 * N], p0);
+    sF[1][2][node] = fx_repack(fx_int(f));
+    const int k = min(x.k, 63);
+    f = FxAcc();
+    fx_mac(f, ln[LN_S11 * N], p1);
+    fx_mac(f, ln[LN_S12 * N], p2);
+    fx_mac(f, ln[LN_S10 * N], p0);
+    s1 = fx_int(f) >> k;
+    f = FxAcc();
+    fx_mac(f, ln[LN_S21 * N], p1);
+    fx_mac(f, ln[LN_S22 * N], p2);
+    fx_mac(f, ln[LN_S20 * N], p0);
+    s2 = fx_int(f) >> k;
+#pragma unroll
+    for (int i = 0; i < TanPoint<NS>::EC; ++i) {
+      const int r = node + i * NN;
+      if (r < 12 * NS) sB[r] = fx_pack(pt.e[i], (r / NS) % 3 == 0 ? E0 : TF);
+    }
+    return;
+  }
+  // the element keeps FP64 values: its coefficients unpacked (or, where the
+  // linearisation left them so, as they are)
+  auto coef = [&](int i, int E) { return x.packed ? fx_unpack(ln[i * N], E) : ln[i * N]; };
+  const int es = De + x.u - x.k, es0 = De + x.a - x.k;
+  const double u1 = coef(LN_U1, x.u), u2 = coef(LN_U2, x.u);
+  const double f12 = fma(u2, pt.v1, fma(u1, pt.v2, coef(LN_A12, x.a) * pt.v0));
+  sF[0][0][node] = pt.v1;
+  sF[1][0][node] = pt.v2;
+  sF[0][1][node] = fma(2.0 * u1, pt.v1, coef(LN_A11, x.a) * pt.v0);
+  sF[0][2][node] = f12;
+  sF[1][1][node] = f12;
+  sF[1][2][node] = fma(2.0 * u2, pt.v2, coef(LN_A22, x.a) * pt.v0);
+  s1 = __double_as_longlong(fma(coef(LN_S11, es), pt.v1, fma(coef(LN_S12, es), pt.v2, coef(LN_S10, es0) * pt.v0)));
+  s2 = __double_as_longlong(fma(coef(LN_S21, es), pt.v1, fma(coef(LN_S22, es), pt.v2, coef(LN_S20, es0) * pt.v0)));
+#pragma unroll
+  for (int i = 0; i < TanPoint<NS>::EC; ++i) {
+    const int r = node + i * NN;
+    if (r < 12 * NS) sB[r] = pt.e[i];
+  }
+}
+
+// the sweeps of the split product with the element's keys M0, t and sources s1, s2
+template <int NS>
+__device__ __forceinline__ void tan_sweep(const double (*sF)[3][NS * NS], const double* sB, int k1, int k2,
+                                          const double* Da, const double* Db, const DfrConst& dc, double dscale,
+                                          bool fixed, unsigned M0, unsigned t, long long s1, long long s2,
+                                          double res[3]) {
+  const int TF = t == 0u ? 1023 : (int)t - 1020;
+  const double add1 = fixed ? 0.0 : dscale * __longlong_as_double(s1);
+  const double add2 = fixed ? 0.0 : dscale * __longlong_as_double(s2);
+  fx_sweep<NS, false>(sF, sB, k1, k2, Da, Db, dc, dscale, fixed, fx_exp(M0), TF, s1, s2, add1, add2, res);
 }
 
 // the two DFR sweeps of one node (rows Da, Db of the scaled derivative
@@ -390,29 +524,27 @@ __device__ __forceinline__ void volume_tangent_body(const TanVolArgs<T>& a, cons
   const int k2 = node / NS, k1 = node % NS;
   const long long idx = elem * NN + node;
   const double dscale = -dc.two_over_dx * a.ep.scale;
-  FxPoint<NS> pt;
-  double S1 = 0.0, S2 = 0.0;
+  TanPoint<NS> pt;
+  LinExp x{};
   unsigned m0 = 0u, m1 = 0u;
   if (active) {
-    tan_fluxes<NS>(a, idx, pt, S1, S2);
-    fx_edges<NS>(a.fb, elem, node, pt, m0, m1);
+    x = lin_exp(a.le, elem);
+    tan_load<NS>(a, elem, node, idx, x, pt, m0, m1);
   }
   __syncthreads();
   fx_block_max<NN, EPB, BLOCK>(sm.sE[0], le, m0, m1);
   __syncthreads();
   bool fixed = false;
+  long long s1 = 0, s2 = 0;
   if (active) {
     m0 = sm.sE[0][le][0];
     m1 = sm.sE[0][le][1];
-    fixed = fx_usable(m0) && fx_usable(m1) && fx_scale_usable(dscale);
-    fx_store<NS>(sm.sF[le], &sm.sB[le][0][0][0], node, pt, fixed, m0, m1);
+    fixed = x.packed && fx_usable(m0) && fx_bid_usable(m1) && fx_scale_usable(dscale);
+    tan_fluxes<NS>(a, sm.sF[le], &sm.sB[le][0][0][0], node, idx, x, pt, dc.dq_exp + 1080, fixed, m0, m1, s1, s2);
   }
   __syncthreads();
   double res[3] = {0.0, 0.0, 0.0};
-  if (active) {
-    fx_sweep<NS>(sm.sF[le], &sm.sB[le][0][0][0], k1, k2, sm.sD[k1], sm.sD[k2], dc, dscale, fixed, m0, m1, a.ep.scale * S1,
-                 a.ep.scale * S2, res);
-  }
+  if (active) tan_sweep<NS>(sm.sF[le], &sm.sB[le][0][0][0], k1, k2, sm.sD[k1], sm.sD[k2], dc, dscale, fixed, m0, m1, s1, s2, res);
   volume_epilogue<BLOCK, true, W3, !F32>(a.ep, active, idx, a.nodes, res, a.out, blk, nblk);
 }
 
@@ -471,29 +603,30 @@ __device__ __forceinline__ void volume_tangent_persistent(const TanVolArgs<T>& a
       const long long elem = eb + le;
       const bool active = lane_on && elem < e1;
       const long long idx = elem * NN + node;
-      FxPoint<NS> pt;
-      double S1 = 0.0, S2 = 0.0;
+      TanPoint<NS> pt;
+      LinExp x{};
       unsigned m0 = 0u, m1 = 0u;
       if (active) {
-        tan_fluxes<NS>(a, idx, pt, S1, S2);
-        fx_edges<NS>(a.fb, elem, node, pt, m0, m1);
+        x = lin_exp(a.le, elem);
+        tan_load<NS>(a, elem, node, idx, x, pt, m0, m1);
       }
       // this parity's keys were zeroed before the previous tile's last barrier
       fx_block_max<NN, EPB, BLOCK>(sm.sE[par], le, m0, m1);
       __syncthreads();   // the keys are complete; the previous tile's readers are done with sF and sB
       bool fixed = false;
+      long long s1 = 0, s2 = 0;
       if (active) {
         m0 = sm.sE[par][le][0];
         m1 = sm.sE[par][le][1];
-        fixed = scale_ok && fx_usable(m0) && fx_usable(m1);
-        fx_store<NS>(sm.sF[le], &sm.sB[le][0][0][0], node, pt, fixed, m0, m1);
+        fixed = x.packed && scale_ok && fx_usable(m0) && fx_bid_usable(m1);
+        tan_fluxes<NS>(a, sm.sF[le], &sm.sB[le][0][0][0], node, idx, x, pt, dc.dq_exp + 1080, fixed, m0, m1, s1, s2);
       }
       for (int t = threadIdx.x; t < 2 * EPB; t += BLOCK) sm.sE[par ^ 1][t >> 1][t & 1] = 0u;
       __syncthreads();
       if (active) {
         double res[3];
-        fx_sweep<NS>(sm.sF[le], &sm.sB[le][0][0][0], k1, k2, sm.sD[k1], sm.sD[k2], dc, dscale, fixed, m0, m1, a.ep.scale * S1,
-                     a.ep.scale * S2, res);
+        tan_sweep<NS>(sm.sF[le], &sm.sB[le][0][0][0], k1, k2, sm.sD[k1], sm.sD[k2], dc, dscale, fixed, m0, m1, s1, s2,
+                      res);
         epilogue_node<W3, !F32>(a.ep, coef, idx, a.nodes, res, a.out, da, db, dcc, dab, dbc);
       }
     }

@@ -408,7 +408,7 @@ int launch_tile(Ctx& c, const double* v, double* out, const AugEpilogue& ep, cud
   using L = TileLayout<NS, DOTS>;
   auto kernel = volume_tangent_tile_f32_kernel<NS, W3, DOTS>;
   if (int rc = set_tile_smem<NS, W3, false, DOTS>()) return rc;
-  TanVolArgs<float> va{v, c.nodes, c.nelem, c.d_lin_node32, reinterpret_cast<const float*>(c.d_fb), out, ep};
+  TanVolArgs<float> va{v, c.nodes, c.nelem, c.d_lin_node32, nullptr, reinterpret_cast<const float*>(c.d_fb), out, ep};
   const long long tiles = (c.nodes + TileShape<NS>::TN - 1) / TileShape<NS>::TN;
   const int ctas = persistent_ctas(c, tiles, tile_ctas_per_sm<DOTS>());
   if (ctas < 0) return SW_ECUDA;
@@ -454,7 +454,7 @@ int capture_volume_tile_dev(Ctx& c, KDev* kd, const KFix& f, bool w3, cudaStream
   if ((f.n * sizeof(float)) % 16 != 0) return 1;
   using L = TileLayout<NS, false>;
   if (int rc = set_tile_smem<NS, false, true, false>()) return rc;
-  TanVolArgs<float> va{nullptr, c.nodes, c.nelem, c.d_lin_node32, reinterpret_cast<const float*>(c.d_fb), nullptr,
+  TanVolArgs<float> va{nullptr, c.nodes, c.nelem, c.d_lin_node32, nullptr, reinterpret_cast<const float*>(c.d_fb), nullptr,
                        AugEpilogue{}};
   const long long tiles = (c.nodes + TileShape<NS>::TN - 1) / TileShape<NS>::TN;
   const int ctas = persistent_ctas(c, tiles, tile_ctas_per_sm<false>());

@@ -67,6 +67,7 @@ struct EnsDesc {
   const double* fc;
   const double* lf;
   const double* ln;
+  const int4* le;
   double* fb;
   double* V;
   long long ldv;
@@ -229,7 +230,7 @@ __device__ __forceinline__ void vol_range(const EnsDesc& d, int j, unsigned int 
   // memory: read where used instead of held in registers through the body
   __shared__ TanVolArgs<double> sva;
   if (threadIdx.x == 0)
-    sva = TanVolArgs<double>{d.V + (long long)j * d.ldv, d.nodes, d.nelem, d.ln, d.fb,
+    sva = TanVolArgs<double>{d.V + (long long)j * d.ldv, d.nodes, d.nelem, d.ln, d.le, d.fb,
                              d.V + (long long)(j + 1) * d.ldv, iter_epilogue(d, j)};
   __syncthreads();
   const TanVolArgs<double>& va = sva;
@@ -1081,6 +1082,7 @@ int ens_run(Ens& e, int steps, const int* orders, const double* dts, double* con
     EnsDesc& d = e.hdesc[m];
     d.lf = c.d_lin_face;
     d.ln = c.d_lin_node;
+    d.le = c.d_lin_exp;
     if ((rc = upload_desc(e, m, s))) return rc;
   }
   long long live_nodes = 0;
@@ -1214,6 +1216,7 @@ int ens_tune(Ens& e, double* const* q, int iters, cudaStream_t s, int* chosen_bl
     d.flags = c.d_flags;
     d.lf = c.d_lin_face;
     d.ln = c.d_lin_node;
+    d.le = c.d_lin_exp;
     d.tol = 0.0;
     d.scale = 1.0;
     d.nu = 0.0;

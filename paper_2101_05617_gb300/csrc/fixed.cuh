@@ -62,6 +62,12 @@ __device__ __forceinline__ double fx_pack(double x, int E) {
   return __hiloint2double(((int)xh ^ s) - s, ((int)xl ^ s) - s);
 }
 
+// the FP64 value of a packed one (rounded to 53 bits)
+__device__ __forceinline__ double fx_unpack(double p, int E) {
+  const double x = fma((double)__double2hiint(p), 536870912.0, (double)__double2loint(p));
+  return x * __hiloint2double((E - 57) << 20, 0);   // 2^(E - 1080)
+}
+
 // sum of products of packed values
 struct FxAcc {
   long long hh = 0, mid = 0;
@@ -75,6 +81,14 @@ __device__ __forceinline__ void fx_mac(FxAcc& a, double x, double m) {
 // the sum in units of 2^58 times the product of the two blocks' units
 __device__ __forceinline__ double fx_sum(const FxAcc& a) {
   return (double)(a.hh + ((a.mid + (1ll << (kFxLimb - 1))) >> kFxLimb));
+}
+
+// the same sum as an integer, and as a packed value (|sum| < 2^58)
+__device__ __forceinline__ long long fx_int(const FxAcc& a) {
+  return a.hh + ((a.mid + (1ll << (kFxLimb - 1))) >> kFxLimb);
+}
+__device__ __forceinline__ double fx_repack(long long y) {
+  return __hiloint2double((int)(y >> kFxLimb), (int)y & 0x1fffffff);
 }
 
 // s 2^k for an integer-valued s (a converted sum), through the exponent field

@@ -134,7 +134,8 @@ struct Ctx {
   // split JVP (dfr_split.cu): coefficients of the imaginary half at the last linearisation point
   int jvp_mode = 1;                 // 0 = plain complex-step evaluation per JVP, 1 = split, 2 = split FP32 bulk
   bool linearized = false;
-  double* d_lin_node = nullptr;     // [LN_COUNT][nodes]
+  double* d_lin_node = nullptr;     // [LN_COUNT][nodes], packed (lin_node_kernel)
+  int4* d_lin_exp = nullptr;        // their exponents per element
   double* d_lin_face = nullptr;     // [18][nfacepts]
   float* d_lin_node32 = nullptr;    // FP32 copies (complex64-bulk form)
   float* d_lin_face32 = nullptr;    // [23][nfacepts]: the 18 flux-map rows, then M00, M01, M10, M11, sigma
