@@ -506,60 +506,18 @@ __device__ __forceinline__ void tile_coef32(const AugEpilogue& ep, float* coef32
   }
 }
 
-// imaginary half of EPB elements per block: block blk of nblk working on one
-// grid; the block has BLOCK >= EPB * NS^2 threads (one per solution point, the
-// rest idle), all of which call this function
-template <typename T, int NS, int EPB, int BLOCK = EPB * NS * NS, bool W3 = false>
-__device__ __forceinline__ void volume_tangent_body(const TanVolArgs<T>& a, const DfrConst& dc, unsigned int blk,
-                                                    unsigned int nblk, VolSmem<T, NS, EPB>& sm) {
-  constexpr int NN = NS * NS;
-  constexpr bool F32 = sizeof(T) == 4;
-  static_assert(EPB * NN <= BLOCK, "block too small for the element tile");
-  static_assert(!F32, "the batched kernels run in FP64");
-  tile_dmat<T, NS, EPB, BLOCK>(a, dc, sm);
-  for (int t = threadIdx.x; t < 2 * EPB; t += BLOCK) sm.sE[0][t >> 1][t & 1] = 0u;
-  const int le = threadIdx.x / NN, node = threadIdx.x % NN;
-  const long long elem = (long long)blk * EPB + le;
-  const bool active = threadIdx.x < EPB * NN && elem < a.nelem;
-  const int k2 = node / NS, k1 = node % NS;
-  const long long idx = elem * NN + node;
-  const double dscale = -dc.two_over_dx * a.ep.scale;
-  TanPoint<NS> pt;
-  LinExp x{};
-  unsigned m0 = 0u, m1 = 0u;
-  if (active) {
-    x = lin_exp(a.le, elem);
-    tan_load<NS>(a, elem, node, idx, x, pt, m0, m1);
-  }
-  __syncthreads();
-  fx_block_max<NN, EPB, BLOCK>(sm.sE[0], le, m0, m1);
-  __syncthreads();
-  bool fixed = false;
-  long long s1 = 0, s2 = 0;
-  if (active) {
-    m0 = sm.sE[0][le][0];
-    m1 = sm.sE[0][le][1];
-    fixed = x.packed && fx_usable(m0) && fx_bid_usable(m1) && fx_scale_usable(dscale);
-    tan_fluxes<NS>(a, sm.sF[le], &sm.sB[le][0][0][0], node, idx, x, pt, dc.dq_exp + 1080, fixed, m0, m1, s1, s2);
-  }
-  __syncthreads();
-  double res[3] = {0.0, 0.0, 0.0};
-  if (active) tan_sweep<NS>(sm.sF[le], &sm.sB[le][0][0][0], k1, k2, sm.sD[k1], sm.sD[k2], dc, dscale, fixed, m0, m1, s1, s2, res);
-  volume_epilogue<BLOCK, true, W3, !F32>(a.ep, active, idx, a.nodes, res, a.out, blk, nblk);
-}
-
-// The same imaginary half as a persistent grid: CTA b of the grid takes the
-// elements [E b / G, E (b + 1) / G) (E elements, G CTAs) in tiles of EPB, adds
-// its window-dot terms up across its tiles and reduces them once.  The even
-// split keeps the last tiles from running on a few SMs alone; the single
-// reduction per CTA saves the per-tile block sums (FP64 adds on the slow pipe).
+// The imaginary half of the elements e0 .. e1 - 1 of one grid in tiles of EPB
+// elements, by a block of BLOCK >= EPB * NS^2 threads (one per solution point, the
+// rest idle), all of which call this function: share blk of nblk of the grid's
+// volume work.  The window-dot terms are added up across the tiles and reduced
+// once per share (per-tile block sums are FP64 adds on the slow pipe).
 template <typename T, int NS, int EPB, int BLOCK, bool W3>
-__device__ __forceinline__ void volume_tangent_persistent(const TanVolArgs<T>& a, const DfrConst& dc,
-                                                          VolSmem<T, NS, EPB>& sm) {
+__device__ __forceinline__ void volume_tangent_range(const TanVolArgs<T>& a, const DfrConst& dc,
+                                                     VolSmem<T, NS, EPB>& sm, long long e0, long long e1,
+                                                     unsigned int blk, unsigned int nblk) {
   constexpr int NN = NS * NS;
   constexpr bool F32 = sizeof(T) == 4;
   static_assert(EPB * NN <= BLOCK, "block too small for the element tile");
-  const long long e0 = a.nelem * blockIdx.x / gridDim.x, e1 = a.nelem * (blockIdx.x + 1) / gridDim.x;
   tile_dmat<T, NS, EPB, BLOCK>(a, dc, sm);
   __shared__ double coef[MAX_NB];
   __shared__ float coef32[MAX_NB];
@@ -632,7 +590,17 @@ __device__ __forceinline__ void volume_tangent_persistent(const TanVolArgs<T>& a
     }
   }
   __shared__ double sred[(W3 ? 5 : 3) * BLOCK];
-  epilogue_finish<BLOCK, W3>(a.ep, da, db, dcc, blockIdx.x, gridDim.x, dab, dbc, sred);
+  epilogue_finish<BLOCK, W3>(a.ep, da, db, dcc, blk, nblk, dab, dbc, sred);
+}
+
+// The same as a persistent grid: CTA b of G takes the elements [E b / G, E (b +
+// 1) / G) of E.  The even split keeps the last tiles from running on a few SMs
+// alone.
+template <typename T, int NS, int EPB, int BLOCK, bool W3>
+__device__ __forceinline__ void volume_tangent_persistent(const TanVolArgs<T>& a, const DfrConst& dc,
+                                                          VolSmem<T, NS, EPB>& sm) {
+  volume_tangent_range<T, NS, EPB, BLOCK, W3>(a, dc, sm, a.nelem * blockIdx.x / gridDim.x,
+                                              a.nelem * (blockIdx.x + 1) / gridDim.x, blockIdx.x, gridDim.x);
 }
 
 }  // namespace swepi

@@ -10,7 +10,7 @@
 // the face kernel), the FP32 b-column copies of the augmented operator and the
 // FP64 orthogonalisation window vectors -- so that all of a tile's HBM traffic
 // is in flight at once; the threads then compute from shared memory exactly
-// what volume_tangent_body computes (pointwise imaginary fluxes and sources,
+// what volume_tangent_range computes (pointwise imaginary fluxes and sources,
 // the DFR sweeps of Eq. 12-14, the augmented operator, the window dots of the
 // incomplete orthogonalisation) and share its epilogue.
 //

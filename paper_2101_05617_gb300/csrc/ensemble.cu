@@ -235,12 +235,9 @@ __device__ __forceinline__ void vol_range(const EnsDesc& d, int j, unsigned int 
   __syncthreads();
   const TanVolArgs<double>& va = sva;
   auto& sm = *reinterpret_cast<VolSmem<double, NS, EPB>*>(smem);
-  for (int k = 0; k < d.vol_tiles; ++k) {
-    const unsigned int tile = local * d.vol_tiles + k;
-    if (tile >= d.n_tiles) break;
-    if (k > 0) __syncthreads();
-    volume_tangent_body<double, NS, EPB, BLOCK>(va, d.dc, tile, d.n_tiles, sm);
-  }
+  const long long e0 = (long long)local * d.vol_tiles * EPB;
+  volume_tangent_range<double, NS, EPB, BLOCK, false>(va, d.dc, sm, e0, min(e0 + (long long)d.vol_tiles * EPB, d.nelem),
+                                                      local, d.n_vol);
 }
 
 template <int BLOCK>
@@ -550,7 +547,12 @@ int block_index(int block) {
   return -1;
 }
 
-sw_ens_tiles default_tiles(int block) { return sw_ens_tiles{2 * block, 1, 16 * block}; }
+// Untuned tiles.  One member of each of twelve (n_e, p) classes, 256 threads, an
+// iteration: 179 us; with 16 / 4 vector entries a thread 185 / 202; at 16 entries
+// with one / four volume tiles a task 202 / 193, with 1 / 4 / 8 interface points a
+// thread 190 / 195 / 220 (a task's waits and sums weigh against CTAs idle at a
+// phase's end).
+sw_ens_tiles default_tiles(int block) { return sw_ens_tiles{2 * block, 2, 8 * block}; }
 
 bool tiles_valid(const sw_ens_tiles& t) {
   return t.face_pts >= 32 && t.face_pts <= (1 << 20) && t.vol_tiles >= 1 && t.vol_tiles <= 64 && t.vec_len >= 128 &&
@@ -1239,7 +1241,7 @@ int ens_tune(Ens& e, double* const* q, int iters, cudaStream_t s, int* chosen_bl
   for (int block : kBlocks) {
     if ((rc = ensure_graph(e, block))) return rc;
     e.block = block;
-    for (int m = 0; m < e.count; ++m) e.mem[m].tiles = default_tiles(block);
+    for (int m = 0; m < e.count; ++m) e.mem[m].tiles = sw_ens_tiles{2 * block, 2, 16 * block};   // of the searched set
     for (int m = 0; m < e.count; ++m)
       if ((rc = upload_desc(e, m, s))) return rc;
     for (const std::vector<int>& members : order) {
