@@ -405,7 +405,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) ens_iter_kernel(const Ens
 }
 
 // ---- batched exponential (one CTA per member, then one launch per product)
-__global__ void ens_expm_prep_kernel(const ExpmJob* __restrict__ jobs) {
+__global__ void __launch_bounds__(kExpmPrepThreads) ens_expm_prep_kernel(const ExpmJob* __restrict__ jobs) {
   const ExpmJob& jb = jobs[blockIdx.x];
   expm_prep_body(jb.H, jb.ldh, jb.j, jb.tau, jb.tau_happy, jb.flags, jb.ws, jb.stat);
 }
@@ -413,19 +413,19 @@ __global__ void ens_expm_prep_kernel(const ExpmJob* __restrict__ jobs) {
 __global__ void __launch_bounds__(64) ens_expm_gemm_kernel(const ExpmJob* __restrict__ jobs, int sc, int sa, int sb,
                                                            MatEpi e, int scaling) {
   const ExpmJob& jb = jobs[blockIdx.z];
-  const int r = blockIdx.y * 8 + threadIdx.y, c = blockIdx.x * 8 + threadIdx.x;
-  if (r >= jb.N || c >= jb.N) return;
+  const int r0 = blockIdx.y * 8, c0 = blockIdx.x * 8;
+  if (r0 >= jb.N || c0 >= jb.N) return;   // uniform over the block
   if (scaling) e.alpha = ldexp(1.0, -jb.sq);
-  expm_gemm_entry(jb.ws, jb.N, sc, sa, sb, e, r, c);
+  expm_gemm_tile(jb.ws, jb.N, sc, sa, sb, e, r0, c0);
 }
 
 __global__ void __launch_bounds__(64) ens_expm_square_kernel(const ExpmJob* __restrict__ jobs, int q) {
   const ExpmJob& jb = jobs[blockIdx.z];
-  const int r = blockIdx.y * 8 + threadIdx.y, c = blockIdx.x * 8 + threadIdx.x;
-  if (q >= jb.sq || r >= jb.N || c >= jb.N) return;
+  const int r0 = blockIdx.y * 8, c0 = blockIdx.x * 8;
+  if (q >= jb.sq || r0 >= jb.N || c0 >= jb.N) return;   // uniform over the block
   const MatEpi none{0, 0, 0, 0, -1, -1, -1, 1.0};
   const int src = expm_square_src(q);
-  expm_gemm_entry(jb.ws, jb.N, expm_square_dst(q), src, src, none, r, c);
+  expm_gemm_tile(jb.ws, jb.N, expm_square_dst(q), src, src, none, r0, c0);
 }
 
 __global__ void ens_expm_finish_kernel(const ExpmJob* __restrict__ jobs) {
@@ -996,7 +996,7 @@ int launch_prep_batch(Ens& e, std::vector<ExpmJob>& jobs, std::vector<int>& ids,
   if (jobs.empty()) return SW_OK;
   int rc = upload(e, e.d_jobs, jobs.data(), sizeof(ExpmJob) * jobs.size(), s);
   if (rc) return rc;
-  ens_expm_prep_kernel<<<(unsigned)jobs.size(), 256, 0, s>>>(e.d_jobs);
+  ens_expm_prep_kernel<<<(unsigned)jobs.size(), kExpmPrepThreads, 0, s>>>(e.d_jobs);
   e.st.launches++;
   return cuda_rc(cudaGetLastError());
 }

@@ -174,7 +174,7 @@ __global__ void kg_advance_kernel(KDev* kd, KFix f, cudaGraphConditionalHandle h
   cudaGraphSetConditional(hi, go ? 1u : 0u);
 }
 
-__global__ void kg_expm_prep_kernel(KDev* kd, KFix f, cudaGraphConditionalHandle hq) {
+__global__ void __launch_bounds__(kExpmPrepThreads) kg_expm_prep_kernel(KDev* kd, KFix f, cudaGraphConditionalHandle hq) {
   if (kd->err) {
     if (threadIdx.x == 0) {
       kd->N = 0;
@@ -205,20 +205,20 @@ __global__ void kg_expm_prep_kernel(KDev* kd, KFix f, cudaGraphConditionalHandle
 __global__ void __launch_bounds__(64) kg_expm_gemm_kernel(const KDev* __restrict__ kd, KFix f, ExpmProduct pr,
                                                           int scaling) {
   const int N = kd->N;
-  const int r = blockIdx.y * 8 + threadIdx.y, c = blockIdx.x * 8 + threadIdx.x;
-  if (N < 2 || r >= N || c >= N) return;
+  const int r0 = blockIdx.y * 8, c0 = blockIdx.x * 8;
+  if (N < 2 || r0 >= N || c0 >= N) return;   // uniform over the block
   MatEpi e = pr.e;
   if (scaling) e.alpha = ::ldexp(1.0, -kd->sq);
-  expm_gemm_entry(f.ws, N, pr.c, pr.a, pr.b, e, r, c);
+  expm_gemm_tile(f.ws, N, pr.c, pr.a, pr.b, e, r0, c0);
 }
 
 __global__ void __launch_bounds__(64) kg_expm_square_kernel(const KDev* __restrict__ kd, KFix f) {
   const int N = kd->N, q = kd->sq_i;
-  const int r = blockIdx.y * 8 + threadIdx.y, c = blockIdx.x * 8 + threadIdx.x;
-  if (N < 2 || q >= kd->sq || r >= N || c >= N) return;
+  const int r0 = blockIdx.y * 8, c0 = blockIdx.x * 8;
+  if (N < 2 || q >= kd->sq || r0 >= N || c0 >= N) return;   // uniform over the block
   const MatEpi none{0, 0, 0, 0, -1, -1, -1, 1.0};
   const int src = expm_square_src(q);
-  expm_gemm_entry(f.ws, N, expm_square_dst(q), src, src, none, r, c);
+  expm_gemm_tile(f.ws, N, expm_square_dst(q), src, src, none, r0, c0);
 }
 
 __global__ void kg_sq_advance_kernel(KDev* kd, cudaGraphConditionalHandle hq) {
@@ -400,7 +400,7 @@ int build(Ctx& c, KGraph& G, int p, int iop, bool fp32, int mmax) {
   ExpmProduct pr[8];
   expm_products(0, pr);   // the scaling 2^-s of the first product is applied on the device
   rc = capture_into(attempt, a, G.cap, [&](cudaStream_t s) {
-    kg_expm_prep_kernel<<<1, 256, 0, s>>>(kd, f, hq);
+    kg_expm_prep_kernel<<<1, kExpmPrepThreads, 0, s>>>(kd, f, hq);
     for (int k = 0; k < 8; ++k) kg_expm_gemm_kernel<<<eg, eb, 0, s>>>(kd, f, pr[k], k == 0 ? 1 : 0);
     return cuda_status(cudaGetLastError());
   });

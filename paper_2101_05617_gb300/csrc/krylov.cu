@@ -126,7 +126,7 @@ __global__ void combine_kernel(double* __restrict__ X, const double* __restrict_
 
 // ------------------------------------------------------------ expm
 // (scheme and workspace slots: krylov_device.cuh)
-__global__ void expm_prep_kernel(const double* __restrict__ H, int ldh, int j, double tau, double tau_happy,
+__global__ void __launch_bounds__(kExpmPrepThreads) expm_prep_kernel(const double* __restrict__ H, int ldh, int j, double tau, double tau_happy,
                                  const int* happy, double* A, double* stat) {
   expm_prep_body(H, ldh, j, tau, tau_happy, happy, A, stat);
 }
@@ -134,9 +134,7 @@ __global__ void expm_prep_kernel(const double* __restrict__ H, int ldh, int j, d
 // one product over the whole grid (8 x 8 outputs per block)
 __global__ void __launch_bounds__(64) small_gemm_kernel(double* __restrict__ ws, int N, int sc, int sa, int sb,
                                                         MatEpi e) {
-  const int r = blockIdx.y * 8 + threadIdx.y, c = blockIdx.x * 8 + threadIdx.x;
-  if (r >= N || c >= N) return;
-  expm_gemm_entry(ws, N, sc, sa, sb, e, r, c);
+  expm_gemm_tile(ws, N, sc, sa, sb, e, blockIdx.y * 8, blockIdx.x * 8);
 }
 
 __global__ void expm_finish_kernel(const double* __restrict__ P, int N, double* F, int ldh, double* stat) {
@@ -468,7 +466,7 @@ int launch_expm_prep(Ctx& c, int j, double tau, double tau_happy, cudaStream_t s
     e1 = prof_event(c);
     cudaEventRecord(e0, s);
   }
-  expm_prep_kernel<<<1, 256, 0, s>>>(c.d_H, c.ldh, j, tau, tau_happy, c.d_flags, c.d_expm_ws, c.d_scal + 8);
+  expm_prep_kernel<<<1, kExpmPrepThreads, 0, s>>>(c.d_H, c.ldh, j, tau, tau_happy, c.d_flags, c.d_expm_ws, c.d_scal + 8);
   if (prof_on(c, PK_EXPM)) {
     cudaEventRecord(e1, s);
     prof_record(c, PK_EXPM, e0, e1);

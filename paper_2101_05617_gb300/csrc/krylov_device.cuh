@@ -633,25 +633,36 @@ inline __host__ __device__ int expm_square_dst(int q) { return (q % 2 == 0) ? XS
 // slot holding exp(A) after s squarings
 inline __host__ __device__ int expm_result_slot(int sq) { return expm_square_src(sq); }
 
-// one block: build A (dense, leading dimension N) in slot XS_A and its
-// 1-norm; stat[1] = j used, stat[2] = t, stat[4] = h_{j+1,j}, stat[5] = ||A||_1
+// one block (kExpmPrepThreads): build A (dense, leading dimension N) in slot XS_A
+// and its 1-norm; stat[1] = j used, stat[2] = t, stat[4] = h_{j+1,j}, stat[5] =
+// ||A||_1.  The column sums read H again, sixteen rows in flight (one row after
+// another from A took 53 us at N = 129).
+constexpr int kExpmPrepThreads = 1024;
 __device__ __forceinline__ void expm_prep_body(const double* __restrict__ H, int ldh, int j, double tau,
                                                double tau_happy, const int* happy, double* A, double* stat) {
   const int jj = happy[0] ? happy[1] : j;
   const double t = happy[0] ? tau_happy : tau;
   const int N = jj + 1;
-  for (int i = threadIdx.x; i < N * N; i += blockDim.x) {
-    int r = i / N, c = i % N;
+  auto entry = [&](int r, int c) {
     double v = 0.0;
     if (r < jj && c < jj) v = H[(long long)r * ldh + c];
     else if (r == 0 && c == jj) v = 1.0;
-    A[i] = t * v;
-  }
-  __syncthreads();
+    return t * v;
+  };
+#pragma unroll 4
+  for (int i = threadIdx.x; i < N * N; i += blockDim.x) A[i] = entry(i / N, i % N);
   __shared__ double colsum[MAX_EXPM];
   for (int c = threadIdx.x; c < N; c += blockDim.x) {
     double sum = 0.0;
-    for (int r = 0; r < N; ++r) sum += fabs(A[r * N + c]);
+    int r = 0;
+    for (; r + 16 <= N; r += 16) {
+      double v[16];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) v[k] = entry(r + k, c);
+#pragma unroll
+      for (int k = 0; k < 16; ++k) sum += fabs(v[k]);
+    }
+    for (; r < N; ++r) sum += fabs(entry(r, c));
     colsum[c] = sum;
   }
   __syncthreads();
@@ -665,15 +676,36 @@ __device__ __forceinline__ void expm_prep_body(const double* __restrict__ H, int
   }
 }
 
-// entry (r, c) of one product in the workspace ws (slots of N x N)
-__device__ __forceinline__ void expm_gemm_entry(double* __restrict__ ws, int N, int sc, int sa, int sb,
-                                                const MatEpi& e, int r, int c) {
+// 8 x 8 entries of one product in the workspace ws (slots of N x N), by a block
+// of 8 x 8 threads (all of which call it): the rows of A and columns of B are
+// copied to shared memory first, all copies in flight at once, then every thread
+// runs its chain of N multiply-adds.  N = 129: 18 -> ~10 us a product, the whole
+// exponential 309 -> 195; the chain alone, 129 FP64 instructions of 64 clocks a
+// warp, is 4.
+__device__ __forceinline__ void expm_gemm_tile(double* __restrict__ ws, int N, int sc, int sa, int sb, const MatEpi& e,
+                                               int r0, int c0) {
+  __shared__ double sA[8][MAX_EXPM + 1], sB[MAX_EXPM][8];
   const long long NN = (long long)N * N;
   const double* A = (sa >= 0) ? ws + sa * NN : nullptr;
   const double* B = (sb >= 0) ? ws + sb * NN : nullptr;
+  const int r = r0 + threadIdx.y, c = c0 + threadIdx.x;
+  if (A && B) {
+    auto copy = [](double* dst, const double* src) {
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                   : "memory");
+    };
+    if (r < N)
+      for (int k = threadIdx.x; k < N; k += 8) copy(&sA[threadIdx.y][k], A + r * N + k);
+    if (c < N)
+      for (int k = threadIdx.y; k < N; k += 8) copy(&sB[k][threadIdx.x], B + k * N + c);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+  }
+  if (r >= N || c >= N) return;
   double s = 0.0;
   if (A && B) {
-    for (int k = 0; k < N; ++k) s = fma(A[r * N + k], B[k * N + c], s);
+#pragma unroll 8
+    for (int k = 0; k < N; ++k) s = fma(sA[threadIdx.y][k], sB[k][threadIdx.x], s);
   } else if (A) {
     s = A[r * N + c];
   } else if (B) {
