@@ -48,6 +48,8 @@ struct FaceArgs {
 
 template <typename T, int NS>
 __global__ void __launch_bounds__(128) face_flux_kernel(FaceArgs a, DfrConst dc) {
+  pdl_wait();
+  pdl_trigger();
   if (a.skip && *a.skip) return;
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= a.nfacepts) return;
@@ -109,6 +111,8 @@ template <typename T, int NS, bool W3 = false>
 __global__ void __launch_bounds__(VolShape<NS>::THREADS) volume_kernel(VolArgs a, DfrConst dc) {
   constexpr int EPB = VolShape<NS>::EPB;
   constexpr int NN = NS * NS;
+  pdl_wait();
+  pdl_trigger();
   if (a.ep.skip && *a.ep.skip) return;
   __shared__ VolSmem<double, NS, EPB> sm;
   for (int t = threadIdx.x; t < NS * (NS + 2); t += blockDim.x) sm.sD[t / (NS + 2)][t % (NS + 2)] = dc.Dq[t / (NS + 2)][t % (NS + 2)];
@@ -186,17 +190,19 @@ static int launch_ns(Ctx& c, const double* q, const double* v, double eps, doubl
     e0 = prof_event(c);
     cudaEventRecord(e0, s);
   }
-  face_flux_kernel<T, NS><<<(unsigned)fblocks, fthreads, 0, s>>>(fa, c.dc);
+  // programmatic dependent launch: the second kernel's launch hides under the first
+  if (launch_pdl(face_flux_kernel<T, NS>, dim3((unsigned)fblocks), dim3(fthreads), s, fa, c.dc) != cudaSuccess)
+    return SW_ECUDA;
   if (pf || pv) {
     e1 = prof_event(c);
     cudaEventRecord(e1, s);
   }
   VolArgs va{q, v, eps, c.nodes, c.nelem, c.d_node_coef, c.d_fb, out, ep};
   long long vblocks = (c.nelem + VolShape<NS>::EPB - 1) / VolShape<NS>::EPB;
-  if (ep.dotC)
-    volume_kernel<T, NS, true><<<(unsigned)vblocks, VolShape<NS>::THREADS, 0, s>>>(va, c.dc);
-  else
-    volume_kernel<T, NS, false><<<(unsigned)vblocks, VolShape<NS>::THREADS, 0, s>>>(va, c.dc);
+  const dim3 vgrid((unsigned)vblocks), vblock(VolShape<NS>::THREADS);
+  const cudaError_t ev = ep.dotC ? launch_pdl(volume_kernel<T, NS, true>, vgrid, vblock, s, va, c.dc)
+                                 : launch_pdl(volume_kernel<T, NS, false>, vgrid, vblock, s, va, c.dc);
+  if (ev != cudaSuccess) return SW_ECUDA;
   if (pv) {
     e2 = prof_event(c);
     cudaEventRecord(e2, s);

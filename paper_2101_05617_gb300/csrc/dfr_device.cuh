@@ -57,19 +57,29 @@ __device__ __forceinline__ T load_state(const double* __restrict__ q, const doub
 
 // ---------------------------------------------------------------- AUSM
 // FP64 divisions and square roots are sequences of many FP64 instructions, so
-// each side takes one square root and the fewest reciprocals (a^d and u^d/a^d;
-// the complex step shares 1/q^0 and 1/a^d between its halves).
-// a^d = sqrt(h^dd g_r H) (App. E) and the Froude number M = u^d / a^d
-__device__ __forceinline__ void speed_mach(double q0, double qd, double ad, double& a, double& M) {
-  a = sqrt(ad * q0);
-  M = qd / (q0 * a);
+// each side takes a single reciprocal square root: with rs = 1 / sqrt(c q^0), c =
+// g_r h^dd / sqrt g, a^d = sqrt(c q^0) = c q^0 rs (corrected to the last bit by
+// one residual), 1 / a^d = rs and 1 / q^0 = c rs^2.
+struct SpeedRoot {
+  double a, ia, r;   // a^d, 1 / a^d, 1 / q^0
+};
+__device__ __forceinline__ SpeedRoot speed_root(double q0, double c) {
+  const double x = c * q0, rs = rsqrt(x);
+  const double s = x * rs;
+  return {fma(0.5 * rs, fma(-s, s, x), s), rs, c * rs * rs};
 }
-__device__ __forceinline__ void speed_mach(cs q0, cs qd, double ad, cs& a, cs& M) {
-  const double s = sqrt(ad * q0.re), is = 1.0 / s, r = 1.0 / q0.re;
-  a = {s, (0.5 * ad) * q0.im * is};
-  const double u = qd.re * r, ui = (qd.im - u * q0.im) * r;
-  const double m = u * is;
-  M = {m, (ui - m * a.im) * is};
+// a^d = sqrt(h^dd g_r H) (App. E) and the Froude number M = u^d / a^d
+__device__ __forceinline__ void speed_mach(double q0, double qd, double c, double& a, double& M) {
+  const SpeedRoot z = speed_root(q0, c);
+  a = z.a;
+  M = qd * (z.r * z.ia);
+}
+__device__ __forceinline__ void speed_mach(cs q0, cs qd, double c, cs& a, cs& M) {
+  const SpeedRoot z = speed_root(q0.re, c);
+  a = {z.a, (0.5 * c) * q0.im * z.ia};
+  const double u = qd.re * z.r, ui = (qd.im - u * q0.im) * z.r;
+  const double m = u * z.ia;
+  M = {m, (ui - m * a.im) * z.ia};
 }
 
 // AUSM interface flux, basic splittings (reading of App. D Eq. 138-139; [41]
@@ -141,9 +151,9 @@ __device__ __forceinline__ void ausm_jacobian_side(const double q[3], int d, dou
 // the square roots and reciprocals.)
 __device__ __forceinline__ void ausm_jacobian(const double qL[3], const double qR[3], int d, double ad, double p1,
                                               double p2, double JL[3][3], double JR[3][3]) {
-  const double rL = 1.0 / qL[0], rR = 1.0 / qR[0];
-  const double aL = sqrt(ad * qL[0]), aR = sqrt(ad * qR[0]);
-  const double gL = rL / aL, gR = rR / aR;   // dM/dq^d
+  const SpeedRoot zL = speed_root(qL[0], ad), zR = speed_root(qR[0], ad);
+  const double aL = zL.a, aR = zR.a, rL = zL.r, rR = zR.r;
+  const double gL = rL * zL.ia, gR = rR * zR.ia;   // dM/dq^d
   const double ML = (d == 1 ? qL[1] : qL[2]) * gL, MR = (d == 1 ? qR[1] : qR[2]) * gR;
   double mp, dmp, bp, dbp, mm, dmm, bm, dbm;
   if (fabs(ML) <= 1.0) {

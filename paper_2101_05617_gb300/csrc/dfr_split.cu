@@ -55,6 +55,8 @@ __global__ void __launch_bounds__(VolShape<NS>::THREADS) lin_node_kernel(const d
                                                                          int4* __restrict__ le,
                                                                          float* __restrict__ ln32) {
   constexpr int NN = NS * NS, EPB = VolShape<NS>::EPB, THREADS = VolShape<NS>::THREADS;
+  pdl_wait();
+  pdl_trigger();
   __shared__ unsigned sE[2][EPB][2];
   for (int t = threadIdx.x; t < 4 * EPB; t += THREADS) (&sE[0][0][0])[t] = 0u;
   const long long i = (long long)blockIdx.x * THREADS + threadIdx.x, N = nodes;
@@ -126,6 +128,8 @@ struct LinFaceArgs {
 
 template <int NS>
 __global__ void __launch_bounds__(128) lin_face_kernel(LinFaceArgs a, DfrConst dc) {
+  pdl_wait();
+  pdl_trigger();
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= a.nfacepts) return;
   const int line = (int)(t / NS), i = (int)(t % NS);
@@ -250,11 +254,14 @@ __global__ void to_float_kernel(const double* __restrict__ src, float* __restric
 template <int NS>
 int linearize_ns(Ctx& c, const double* q, cudaStream_t s) {
   const int th = VolShape<NS>::THREADS;
-  lin_node_kernel<NS><<<(unsigned)((c.nodes + th - 1) / th), th, 0, s>>>(
-      q, c.d_node_coef, c.nodes, -0.5 * c.dx, c.dc.dq_exp + 1080, c.d_lin_node, c.d_lin_exp,
-      c.jvp_mode == 2 ? c.d_lin_node32 : nullptr);
+  if (launch_pdl(lin_node_kernel<NS>, dim3((unsigned)((c.nodes + th - 1) / th)), dim3(th), s, q, c.d_node_coef,
+                 c.nodes, -0.5 * c.dx, c.dc.dq_exp + 1080, c.d_lin_node, c.d_lin_exp,
+                 c.jvp_mode == 2 ? c.d_lin_node32 : static_cast<float*>(nullptr)) != cudaSuccess)
+    return SW_ECUDA;
   LinFaceArgs fa{q, c.nodes, c.d_lines, c.d_face_coef, c.nfacepts, c.d_lin_face};
-  lin_face_kernel<NS><<<(unsigned)((c.nfacepts + 127) / 128), 128, 0, s>>>(fa, c.dc);
+  if (launch_pdl(lin_face_kernel<NS>, dim3((unsigned)((c.nfacepts + 127) / 128)), dim3(128), s, fa, c.dc) !=
+      cudaSuccess)
+    return SW_ECUDA;
   c.launches += 2;
   return cuda_status(cudaGetLastError());
 }

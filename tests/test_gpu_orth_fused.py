@@ -58,3 +58,36 @@ def test_fused_passes_kiops_parity(iop):
     assert max(err) < 1e-10, (err, st, rst)
     assert (st["krylov_iters"], st["substeps"], st["rejects"]) == \
         (rst["krylov_iters"], rst["substeps"], rst["rejects"]), (st, rst)
+
+
+@pytest.mark.parametrize("ne,p", [(66, 5), (14, 3), (1, 1)])
+def test_kept_entries_and_their_remainder(ne, p):
+    """The fused FP64 pass keeps a thread's first 32 entries of z in registers:
+    sizes past that (2.82 M unknowns: 37 a thread), part of a thread's batches,
+    and fewer entries than threads agree bit for bit with the two launches."""
+    from paper_2101_05617_gb300.swepi import SWContext
+    nodes = 6 * ne * ne * (p + 1) ** 2
+    gen = torch.Generator(device="cuda").manual_seed(ne)
+
+    def field(k):
+        x = torch.randn(3 * nodes, generator=gen, device="cuda", dtype=torch.float64)
+        x[:nodes] *= 1e13
+        x[nodes:] *= 1e9
+        return x if k else None
+    b = [field(k) for k in range(3)]
+    out = []
+    for fused in (0, 1):
+        ctx = SWContext(ne, p, (0.3, -0.2, 0.4))
+        assert ctx.set_orth_fused(fused) == fused
+        xyz = torch.tensor(ctx.node_xyz(), device="cuda").reshape(3, -1)
+        q = torch.tensor(ctx.state_from_fields((8000.0 + 50.0 * xyz[2]).cpu().numpy(), [0.0] * nodes,
+                                               (10.0 * torch.stack([-xyz[1], xyz[0], 0 * xyz[0]])).cpu().numpy()),
+                         device="cuda")
+        for iop in (2, 3):
+            w, st = ctx.kiops_phi(q, 30.0, b, tol=1e-6, m_init=12, iop=iop)
+            assert torch.isfinite(w).all()
+            out.append((w.clone(), st))
+        ctx.close()
+    for k in range(2):
+        assert out[k][1] == out[2 + k][1]
+        assert torch.equal(out[k][0], out[2 + k][0])
