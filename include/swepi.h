@@ -202,8 +202,8 @@ int sw_set_jvp_mode(sw_ctx_t ctx, int mode);
 int sw_set_kiops_driver(sw_ctx_t ctx, int driver);
 
 /* The two vector passes of the fused incomplete orthogonalisation (the
- * modified Gram-Schmidt updates with ||z||, then the scaling with the next
- * window dot; the KIOPS reading of Eq. 29's Krylov projection) in one launch:
+ * modified Gram-Schmidt updates with ||z||, then the scaling; the KIOPS reading
+ * of Eq. 29's Krylov projection) in one launch:
  * enable = 1 (default) runs them as one cooperative launch whose CTAs wait on
  * one another for ||z|| (a bounded wait: SW_ETIMEOUT past about a second),
  * where the GPU holds the whole grid at once; 0 = two launches.  The results
@@ -437,7 +437,7 @@ long long sw_kernel_launches(sw_ctx_t ctx);
  * milliseconds since the last sw_profile(ctx, 1).  kind: 0 = face flux (JVP),
  * 1 = volume (JVP), 2 = face flux (RHS), 3 = volume (RHS), 4 = exponential,
  * 5 = linearisation of the split JVP, 6 = the two vector passes of the fused
- * orthogonalisation (update + norm, scale + dot). */
+ * orthogonalisation (update + norm, scale). */
 #define SW_PROF_KINDS 7
 typedef struct {
   long long count[SW_PROF_KINDS];

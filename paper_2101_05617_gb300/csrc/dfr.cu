@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(VolShape<NS>::THREADS) volume_kernel(VolArgs a
       for (int mu = 0; mu < 3; ++mu) res[mu] *= sc;
     }
   }
-  volume_epilogue<VolShape<NS>::THREADS, false, W3>(a.ep, active, idx, a.nodes, res, a.out, blockIdx.x, gridDim.x);
+  volume_epilogue<VolShape<NS>::THREADS, W3>(a.ep, active, idx, a.nodes, res, a.out, blockIdx.x, gridDim.x);
 }
 
 // ---------------------------------------------------------------- launchers

@@ -244,16 +244,13 @@ __device__ __forceinline__ void epilogue_finish(const AugEpilogue& ep, double da
                                                 unsigned int blk, unsigned int nblk, double dab, double dbc,
                                                 double* sbuf);
 
-// Epilogue of the volume kernels (all threads of the block call it; blk/nblk:
-// this block's index and the number of blocks working on the same vector):
-// out = scale * res + nu * sum_l y_l b_{p-l} (the augmented operator of the
-// phi-function solver), the shift of the augmented tail, and -- when dotB is
+// Epilogue of the full-evaluation volume kernels (all threads of the block call
+// it; blk/nblk: this block's index and the number of blocks working on the same
+// vector): out = scale * res + nu * sum_l y_l b_{p-l} (the augmented operator of
+// the phi-function solver), the shift of the augmented tail, and -- when dotB is
 // set -- the window dot products of the incomplete orthogonalisation (two or
-// three vectors; see AugEpilogue).
-// SCALED: the caller has already multiplied res by scale.  W3: compiled for
-// the window of three (dotC may be set); W3 = false drops that code.  B64:
-// the b-column terms are added here in FP64; false: the caller has added them
-// already (the FP32 kernels of the complex64-bulk form, from ep.b32).
+// three vectors; see AugEpilogue).  W3: compiled for the window of three (dotC
+// may be set); W3 = false drops that code.  The tangent kernels call its parts.
 // the tail coefficients nu * y_l of the augmented operator into coef[MAX_NB]
 // (shared memory; the caller synchronises before reading them)
 __device__ __forceinline__ void epilogue_coefs(const AugEpilogue& ep, double* coef) {
@@ -309,19 +306,19 @@ __device__ __forceinline__ void epilogue_node(const AugEpilogue& ep, const doubl
   }
 }
 
-template <int THREADS, bool SCALED = false, bool W3 = false, bool B64 = true>
+template <int THREADS, bool W3>
 __device__ __forceinline__ void volume_epilogue(const AugEpilogue& ep, bool active, long long idx, long long N,
                                                 const double res[3], double* __restrict__ out, unsigned int blk,
                                                 unsigned int nblk) {
   __shared__ double coef[MAX_NB];
-  if (B64) epilogue_coefs(ep, coef);
+  epilogue_coefs(ep, coef);
   __syncthreads();
   double da = 0.0, db = 0.0, dcc = 0.0, dab = 0.0, dbc = 0.0;
   if (active) {
     double r[3];
 #pragma unroll
-    for (int mu = 0; mu < 3; ++mu) r[mu] = SCALED ? res[mu] : ep.scale * res[mu];
-    epilogue_node<W3, B64>(ep, coef, idx, N, r, out, da, db, dcc, dab, dbc);
+    for (int mu = 0; mu < 3; ++mu) r[mu] = ep.scale * res[mu];
+    epilogue_node<W3, true>(ep, coef, idx, N, r, out, da, db, dcc, dab, dbc);
   }
   __shared__ double sred[(W3 ? 5 : 3) * THREADS];
   epilogue_finish<THREADS, W3>(ep, da, db, dcc, blk, nblk, dab, dbc, sred);
