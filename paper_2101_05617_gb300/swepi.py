@@ -186,8 +186,20 @@ def _check(call, rc):
         raise SWError(call, rc)
 
 
+_torch_module = None
+
+
+def _torch():
+    """torch, imported on first use (an import statement in every call costs small calls a microsecond)."""
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
+
+
 def _dev_ptr(t, n=None):
-    import torch
+    torch = _torch()
     if not isinstance(t, torch.Tensor) or not t.is_cuda or t.dtype != torch.float64 or not t.is_contiguous():
         raise TypeError("expected a contiguous float64 CUDA tensor")
     if n is not None and t.numel() < n:
@@ -196,9 +208,10 @@ def _dev_ptr(t, n=None):
 
 
 def _stream(stream):
-    import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return ctypes.c_void_p(stream.cuda_stream)
+    torch = _torch()   # the current stream's handle, without a Stream object around it
+    return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
 
 
 def _host(a, n):
@@ -706,25 +719,26 @@ class SWContext:
         else:
             sw_set_bottom_host(self.handle, np.asarray(hB))
 
+    # the calls of a few microseconds go to the library directly: the context
+    # knows its number of unknowns, which the C-named functions ask for each time
     def rhs(self, q, out=None, stream=None):
-        import torch
-        out = torch.empty_like(q) if out is None else out
-        sw_rhs(self.handle, q, out, stream)
+        out = _torch().empty_like(q) if out is None else out
+        _check("sw_rhs", lib().sw_rhs(self.handle, _dev_ptr(q, self.n), _dev_ptr(out, self.n), _stream(stream)))
         return out
 
     def jvp(self, q, v, eps=1e-30, out=None, stream=None):
-        import torch
-        out = torch.empty_like(q) if out is None else out
-        sw_jvp(self.handle, q, v, eps, out, stream)
+        out = _torch().empty_like(q) if out is None else out
+        _check("sw_jvp", lib().sw_jvp(self.handle, _dev_ptr(q, self.n), _dev_ptr(v, self.n), float(eps),
+                                      _dev_ptr(out, self.n), _stream(stream)))
         return out
 
     def linearize(self, q, stream=None):
-        sw_linearize(self.handle, q, stream)
+        _check("sw_linearize", lib().sw_linearize(self.handle, _dev_ptr(q, self.n), _stream(stream)))
 
     def jvp_linearized(self, v, out=None, stream=None):
-        import torch
-        out = torch.empty_like(v) if out is None else out
-        sw_jvp_linearized(self.handle, v, out, stream)
+        out = _torch().empty_like(v) if out is None else out
+        _check("sw_jvp_linearized", lib().sw_jvp_linearized(self.handle, _dev_ptr(v, self.n), _dev_ptr(out, self.n),
+                                                            _stream(stream)))
         return out
 
     def set_jvp_mode(self, mode):
