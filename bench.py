@@ -51,7 +51,7 @@ def flops_per_jvp(ne, ns, p=4, dots=True):
 # the phi-function solver (p = 4, with dots), from one ncu capture of the
 # kernel as it stands (dram__bytes_read.sum + dram__bytes_write.sum); none
 # while the kernel has changed since its last capture.
-TRAFFIC_BYTES = {"ne60_p5": 187.29e6}   # 174.60 MB read + 12.69 MB written
+TRAFFIC_BYTES = {"ne60_p5": 188.05e6}   # 176.23 MB read + 11.83 MB written
 
 # phi-vectors phi_1 .. phi_M of an EPI order (the b columns of its phi-function call)
 EPI_PHI = {2: 1, 3: 2, 4: 3, 5: 4, 6: 4}
