@@ -45,6 +45,10 @@ namespace {
 // the u^i, a for the A^{ij}, s for the S^i_j, s0 for the S^i_0, with
 //   s0 - s = a - u       (the terms of a source come out in one unit) and
 //   k = De + u - s >= 0  (a source adds to the packed sweep after a right shift).
+// u and a are the classes' own exponents, raised only where a source outweighs
+// the whole sweep (which is then what the sum is rounded against); the S^i_j
+// and S^i_0 take what is left, so the fluxes' coefficients keep their bits
+// however small the sources' are (no Coriolis term at a panel centre).
 // The sources are stored times -dx/2: the sweep's sums and they share the factor
 // -2/dx.  An element with a coefficient past the format's range keeps FP64 values.
 // ln32 (complex64-bulk form): the unscaled coefficients rounded to FP32.
@@ -105,14 +109,14 @@ __global__ void __launch_bounds__(VolShape<NS>::THREADS) lin_node_kernel(const d
   ms = sE[1][e][0];
   ms0 = sE[1][e][1];
   const bool packed = fx_usable(mu) && fx_usable(ma) && fx_usable(ms) && fx_usable(ms0);
-  // an all-zero class takes the smallest exponent and constrains nothing
+  // an all-zero class takes the format's smallest exponent and raises no other
   const int eu = mu ? (int)(mu >> 20) : kFxExpMin, ea = ma ? (int)(ma >> 20) : kFxExpMin;
   const int es = ms ? (int)(ms >> 20) : kFxExpMin, es0 = ms0 ? (int)(ms0 >> 20) : kFxExpMin;
-  const int u = max(eu, es - De), a = max(ea, es0 - es + u), s0 = es + a - u;
-  if (threadIdx.x % NN == 0) le[i / NN] = packed ? make_int4(u, a, De + u - es, 1) : make_int4(0, 0, 0, 0);
+  const int u = max(eu, es - De), a = max(ea, es0 - De), s = max(es, es0 + u - a), s0 = s + a - u;
+  if (threadIdx.x % NN == 0) le[i / NN] = packed ? make_int4(u, a, De + u - s, 1) : make_int4(0, 0, 0, 0);
 #pragma unroll
   for (int k = 0; k < LN_COUNT; ++k) {
-    const int E = k <= LN_U2 ? u : (k <= LN_A22 ? a : ((k == LN_S10 || k == LN_S20) ? s0 : es));
+    const int E = k <= LN_U2 ? u : (k <= LN_A22 ? a : ((k == LN_S10 || k == LN_S20) ? s0 : s));
     ln[k * N + i] = packed ? fx_pack(c[k], E) : c[k];
   }
 }
