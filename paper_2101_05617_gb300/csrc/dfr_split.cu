@@ -108,11 +108,13 @@ __global__ void __launch_bounds__(VolShape<NS>::THREADS) lin_node_kernel(const d
   ma = sE[0][e][1];
   ms = sE[1][e][0];
   ms0 = sE[1][e][1];
-  const bool packed = fx_usable(mu) && fx_usable(ma) && fx_usable(ms) && fx_usable(ms0);
   // an all-zero class takes the format's smallest exponent and raises no other
   const int eu = mu ? (int)(mu >> 20) : kFxExpMin, ea = ma ? (int)(ma >> 20) : kFxExpMin;
   const int es = ms ? (int)(ms >> 20) : kFxExpMin, es0 = ms0 ? (int)(ms0 >> 20) : kFxExpMin;
   const int u = max(eu, es - De), a = max(ea, es0 - De), s = max(es, es0 + u - a), s0 = s + a - u;
+  // v^0 is packed for the exponent t + 2 - a, v^i for t + 2 - u, with t >= 1020 + kFxExpMin: both stay
+  // large enough that a zero or subnormal entry becomes 0 (fx_pack)
+  const bool packed = fx_usable(mu) && fx_usable(ma) && fx_usable(ms) && fx_usable(ms0) && max(u, a) <= kFxCoefMax;
   if (threadIdx.x % NN == 0) le[i / NN] = packed ? make_int4(u, a, De + u - s, 1) : make_int4(0, 0, 0, 0);
 #pragma unroll
   for (int k = 0; k < LN_COUNT; ++k) {

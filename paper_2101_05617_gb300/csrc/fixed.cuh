@@ -27,6 +27,9 @@ namespace swepi {
 constexpr int kFxBits = 58;                      // magnitude bits of a block value
 constexpr int kFxLimb = 29;                      // bits of the low limb
 constexpr int kFxExpMin = 400, kFxExpMax = 1700; // biased exponents of the largest magnitude the format takes
+constexpr int kFxPackMin = 58;                   // smallest block exponent a value is packed for (fx_pack)
+// largest exponent of a packed coefficient class of the split product (lin_node_kernel)
+constexpr int kFxCoefMax = 1020 + kFxExpMin + 2 - kFxPackMin;
 
 // the magnitude key a block's maximum is taken over: the high word without the
 // sign (ordered as the magnitudes are, NaN and infinities above all others)
@@ -49,7 +52,7 @@ __device__ __forceinline__ unsigned shr_clamped(unsigned x, int s) {   // 0 for 
 // x as block value for the block exponent E (>= the exponent of x): h and l
 // packed as the high and low word of a double (a container, never an operand
 // of FP64 arithmetic).  X = trunc(|x| 2^(58 - (E - 1022))), the sign on both
-// limbs.  Zeros and subnormals (exponent field 0, at least 400 below E) become 0.
+// limbs.  Zeros and subnormals (exponent field 0) become 0: E is at least kFxPackMin.
 __device__ __forceinline__ double fx_pack(double x, int E) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const int d = E - (int)((hi >> 20) & 0x7ffu);

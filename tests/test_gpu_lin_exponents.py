@@ -86,3 +86,18 @@ def test_directions_of_one_variable(ne, ns, var):
     for got in _products(g, q, v):
         err = scaled_err_per_var(got, ref, scale)
         assert max(err) < TOL_JVP, err
+
+
+@pytest.mark.parametrize("ns", [2, 5])
+def test_zero_entries_beside_huge_coefficients(ns):
+    """Entries that are zero contribute nothing however large the exponent of
+    their coefficient (a bottom of 1e200 m lifts S^i_0 and with it A) and
+    however small the direction."""
+    _, g, q, _ = oracle_case(2, ns, seed=3)
+    x, y, z = g.node_xyz()
+    hB = 1e200 * (x * y + 0.5 * z)
+    g.set_bottom(hB)
+    v = scaled_direction(q, 5)
+    v[0] = 0.0
+    for k in (0, -260, -320, -340, -360, -400):
+        _check(g, q, np.ldexp(v, k), hB)
