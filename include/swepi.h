@@ -471,7 +471,9 @@ int sw_check_status(int* checked);
 /* Checked builds only (SW_EINVAL otherwise): what = 1 moves the first
  * interface line's owner element one grid past the last element in the
  * context's device table, so that the next face kernel's check fires (the
- * test of the checks); what = 0 moves it back. */
+ * test of the checks); what = 0 moves it back; what = 2 leaves counts in the
+ * phi-function solver's tickets, as a call whose bounded wait gave up can
+ * (SW_EINVAL before the context's first such call). */
 int sw_check_inject(sw_ctx_t ctx, int what);
 
 /* Measured FP64 fused-multiply-add throughput of the current device in

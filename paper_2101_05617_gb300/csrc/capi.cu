@@ -233,8 +233,13 @@ int sw_check_status(int* checked) {
 }
 
 int sw_check_inject(sw_ctx_t c, int what) {
-  if (!c || !kChecked || what < 0 || what > 1) return SW_EINVAL;
+  if (!c || !kChecked || what < 0 || what > 2) return SW_EINVAL;
   if (int rc = check_device(*c)) return rc;
+  if (what == 2) {   // counts no grid of this library reaches
+    if (!c->d_flags) return SW_EINVAL;
+    const int left[3] = {1 << 20, 1 << 20, 1 << 20};
+    return cudaMemcpy(c->d_flags + 8, left, sizeof(left), cudaMemcpyHostToDevice) == cudaSuccess ? SW_OK : SW_ECUDA;
+  }
   FaceLine L;
   if (cudaMemcpy(&L, c->d_lines, sizeof(L), cudaMemcpyDeviceToHost) != cudaSuccess) return SW_ECUDA;
   // 1: the first interface line's owner moved past the last element; 0: moved back

@@ -1076,6 +1076,7 @@ int ens_run(Ens& e, int steps, const int* orders, const double* dts, double* con
     if (cudaStreamWaitEvent(e.mstream[m], e.start_event, 0) != cudaSuccess) return SW_ECUDA;
   for (int m = 0; m < e.count; ++m) {
     if (steps == 0) break;
+    if ((rc = clear_wait_state(*e.mem[m].c, member_stream(e, m)))) return rc;
     // the lin tables are allocated by the first linearisation: start each member, then refresh its tables
     if ((rc = epi_begin_step(e, m, o, s))) return rc;
   }
@@ -1201,7 +1202,7 @@ int ens_tune(Ens& e, double* const* q, int iters, cudaStream_t s, int* chosen_bl
   // a unit start vector per member, lin tables at its state, a plain operator (p = 1, no b)
   for (int m = 0; m < e.count; ++m) {
     Ctx& c = *e.mem[m].c;
-    if ((rc = ensure_krylov(c, 64))) return rc;
+    if ((rc = ensure_krylov(c, 64)) || (rc = clear_wait_state(c, s))) return rc;
     if ((rc = launch_linearize(c, q[m], s))) return rc;
     if ((rc = launch_norm2(c, q[m], c.n, c.d_scal + S_BETA, 0.0, nullptr, 0, nullptr, s))) return rc;
     if ((rc = launch_scale_inv(c, c.d_V, q[m], c.d_scal + S_BETA, c.n, nullptr, s))) return rc;

@@ -86,6 +86,10 @@ int ensure_krylov(Ctx& c, int m_max) {
   return SW_OK;
 }
 
+int clear_wait_state(Ctx& c, cudaStream_t s) {
+  return cuda_status(cudaMemsetAsync(c.d_flags + 3, 0, sizeof(int) * 8, s));
+}
+
 int kiops_run(Ctx& c, const double* q_lin, double dt, double tau_out, int nb, const double* const* b,
               const sw_kiops_opts& o, double* w, sw_kiops_stats* st, cudaStream_t s, bool use_lin) {
   if (nb < 1 || nb > MAX_NB || !(tau_out > 0) || o.m_min < 1 || o.m_max < o.m_min || o.m_max > 150 || o.iop < 1 ||
@@ -102,6 +106,7 @@ int kiops_run(Ctx& c, const double* q_lin, double dt, double tau_out, int nb, co
   if (p == 0) { p = 1; bk[1] = nullptr; }
   const long long N = n + p;
 
+  if ((rc = clear_wait_state(c, s))) return rc;
   // scaling of the augmented operator
   for (int k = 1; k <= p; ++k) {
     if (bk[k]) {
@@ -110,10 +115,6 @@ int kiops_run(Ctx& c, const double* q_lin, double dt, double tau_out, int nb, co
       return SW_ECUDA;
     }
   }
-  if (cudaMemsetAsync(c.d_flags + 3, 0, sizeof(int), s) != cudaSuccess) return SW_ECUDA;
-  // the pass and epilogue tickets and the cooperative passes' barrier counter, in
-  // case a wait that gave up left them mid-count
-  if (cudaMemsetAsync(c.d_flags + 8, 0, sizeof(int) * 3, s) != cudaSuccess) return SW_ECUDA;
   // X = [b_0; 0 .. 0 mu]
   if (bk[0]) {
     if (cudaMemcpyAsync(c.d_X, bk[0], sizeof(double) * n, cudaMemcpyDeviceToDevice, s) != cudaSuccess) return SW_ECUDA;

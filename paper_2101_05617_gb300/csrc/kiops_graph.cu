@@ -499,6 +499,7 @@ int kiops_run_graph(Ctx& c, double dt, double tau_out, int nb, const double* con
   }
   KGraph* G = graph_of(c);
   if (!G) return SW_ENOMEM;
+  if ((rc = clear_wait_state(c, s))) return rc;
   // the 1-norms of b_1..b_p and X = [b_0; 0] (the tail is set on the device)
   for (int k = 1; k <= p; ++k) {
     if (bk[k]) {
@@ -512,7 +513,6 @@ int kiops_run_graph(Ctx& c, double dt, double tau_out, int nb, const double* con
   } else if (cudaMemsetAsync(c.d_X, 0, sizeof(double) * n, s) != cudaSuccess) {
     return SW_ECUDA;
   }
-  if (cudaMemsetAsync(c.d_flags + 3, 0, sizeof(int), s) != cudaSuccess) return SW_ECUDA;
   if (!G->exec || G->p != p || G->iop != o.iop || G->fp32 != (fp32 ? 1 : 0) || G->mmax != o.m_max ||
       G->V != c.d_V || G->V32 != (fp32 ? c.d_V32 : nullptr) || G->b32 != (fp32 ? c.d_b32 : nullptr)) {
     const unsigned prof = c.prof;

@@ -115,7 +115,9 @@ struct Ctx {
   double* d_vpart = nullptr;      // partials of the epilogue dot products (2 per volume block)
   double* d_cdot = nullptr;       // V_j . V_{j-1} per basis index
   double* d_scal = nullptr;       // device scalars (see kiops.cu)
-  int* d_flags = nullptr;         // happy flag, happy size
+  // 0 happy flag, 1 happy size, 3 a bounded wait gave up, 8 ticket of the reductions and vector passes,
+  // 9 ticket of the volume epilogue, 10 counter of the cooperative passes' grid barrier
+  int* d_flags = nullptr;
   double* h_pinned = nullptr;     // pinned read-back area
   const double** d_bptr = nullptr;
   // EPI state
@@ -351,6 +353,10 @@ int launch_lincomb(Ctx& c, double* out, long long n, int k, const double* const*
 int kiops_run(Ctx& c, const double* q_lin, double dt, double tau_out, int nb, const double* const* b,
               const sw_kiops_opts& o, double* w, sw_kiops_stats* st, cudaStream_t s, bool use_lin);
 int ensure_krylov(Ctx& c, int m_max);
+// before a call's first reduction: the gave-up mark, the tickets and the barrier
+// counter, which a call whose bounded wait gave up leaves mid-count (a reduction
+// that starts from such a count never publishes its sum, or does so too early)
+int clear_wait_state(Ctx& c, cudaStream_t s);
 // the device-driven solver (kiops_graph.cu): used by kiops_run when selected and
 // applicable (split JVP, window 2 or 3, plain rule, profiling off)
 bool kiops_graph_applies(const Ctx& c, const sw_kiops_opts& o, bool use_lin);
