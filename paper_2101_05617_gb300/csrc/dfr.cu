@@ -49,7 +49,6 @@ struct FaceArgs {
 template <typename T, int NS>
 __global__ void __launch_bounds__(128) face_flux_kernel(FaceArgs a, DfrConst dc) {
   pdl_wait();
-  pdl_trigger();
   if (a.skip && *a.skip) return;
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= a.nfacepts) return;
@@ -112,7 +111,6 @@ __global__ void __launch_bounds__(VolShape<NS>::THREADS) volume_kernel(VolArgs a
   constexpr int EPB = VolShape<NS>::EPB;
   constexpr int NN = NS * NS;
   pdl_wait();
-  pdl_trigger();
   if (a.ep.skip && *a.ep.skip) return;
   __shared__ VolSmem<double, NS, EPB> sm;
   for (int t = threadIdx.x; t < NS * (NS + 2); t += blockDim.x) sm.sD[t / (NS + 2)][t % (NS + 2)] = dc.Dq[t / (NS + 2)][t % (NS + 2)];
@@ -190,7 +188,12 @@ static int launch_ns(Ctx& c, const double* q, const double* v, double eps, doubl
     e0 = prof_event(c);
     cudaEventRecord(e0, s);
   }
-  // programmatic dependent launch: the second kernel's launch hides under the first
+  // Programmatic dependent launch, triggered by the CTAs' ends alone: a kernel's
+  // launch overlaps its predecessor's last wave.  With the trigger at a kernel's
+  // start its successor's CTAs took their places on SMs while they waited, and on
+  // grids of about one wave the next kernel's CTAs were dealt two to an SM beside
+  // them (6 x 20 x 20, p = 3: right-hand side 23.4 us, full product 38.2; with plain
+  // launches 14.1 and 20.7, like this 13.7 and 19.9; 6 x 60 x 60, p = 5: 96 in all).
   if (launch_pdl(face_flux_kernel<T, NS>, dim3((unsigned)fblocks), dim3(fthreads), s, fa, c.dc) != cudaSuccess)
     return SW_ECUDA;
   if (pf || pv) {

@@ -372,7 +372,8 @@ inline int cuda_status(cudaError_t e) { return e == cudaSuccess ? SW_OK : SW_ECU
 // is still running, so the launch latency between consecutive kernels is
 // hidden.  Each such kernel calls pdl_wait() before its first global memory
 // access of any kind (which returns once the predecessor has completed and its
-// writes are visible) and pdl_trigger() to let its own successor be scheduled.
+// writes are visible).  pdl_trigger() lets a kernel's own successor be scheduled
+// while it runs; without it that happens as its CTAs end (dfr.cu).
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
