@@ -50,7 +50,8 @@ namespace {
 // and S^i_0 take what is left, so the fluxes' coefficients keep their bits
 // however small the sources' are (no Coriolis term at a panel centre).
 // The sources are stored times -dx/2: the sweep's sums and they share the factor
-// -2/dx.  An element with a coefficient past the format's range keeps FP64 values.
+// -2/dx.  An element with a coefficient past the format's range keeps FP64 values,
+// and with N_s = 1 all of them do (volume_tangent_node).
 // ln32 (complex64-bulk form): the unscaled coefficients rounded to FP32.
 template <int NS>
 __global__ void __launch_bounds__(VolShape<NS>::THREADS) lin_node_kernel(const double* __restrict__ q,
@@ -114,7 +115,8 @@ __global__ void __launch_bounds__(VolShape<NS>::THREADS) lin_node_kernel(const d
   const int u = max(eu, es - De), a = max(ea, es0 - De), s = max(es, es0 + u - a), s0 = s + a - u;
   // v^0 is packed for the exponent t + 2 - a, v^i for t + 2 - u, with t >= 1020 + kFxExpMin: both stay
   // large enough that a zero or subnormal entry becomes 0 (fx_pack)
-  const bool packed = fx_usable(mu) && fx_usable(ma) && fx_usable(ms) && fx_usable(ms0) && max(u, a) <= kFxCoefMax;
+  const bool packed = NS > 1 && fx_usable(mu) && fx_usable(ma) && fx_usable(ms) && fx_usable(ms0) &&
+                      max(u, a) <= kFxCoefMax;
   if (threadIdx.x % NN == 0) le[i / NN] = packed ? make_int4(u, a, De + u - s, 1) : make_int4(0, 0, 0, 0);
 #pragma unroll
   for (int k = 0; k < LN_COUNT; ++k) {

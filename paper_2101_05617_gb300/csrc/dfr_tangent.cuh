@@ -506,6 +506,41 @@ __device__ __forceinline__ void tile_coef32(const AugEpilogue& ep, float* coef32
   }
 }
 
+// N_s = 1 in FP64: an element is one node, nothing is shared between threads and
+// each sweep has three terms, so packing 17 values a node and passing them through
+// shared memory (88 bytes of spills, 47 KB) cost more than the 18 multiply-adds:
+// FP64 from registers.  The product at 6 x 16 x 16, p = 0: 10.1 -> 7.8 us (FP64
+// through shared memory 8.7); 6 x 64 x 64: 16.8 -> 10.1; from 6 x 128 x 128 (25.1 us)
+// on it waits for memory either way (6 x 360 x 360: 153 and 156).
+__device__ __forceinline__ void volume_tangent_node(const TanVolArgs<double>& a, const DfrConst& dc, long long elem,
+                                                    double dscale, double res[3]) {
+  const long long N = a.nodes;
+  double e[12];   // interface fluxes [edge][mu], 96 bytes a thread
+#pragma unroll
+  for (int r = 0; r < 6; ++r) {
+    const double2 x = reinterpret_cast<const double2*>(a.fb + elem * 12)[r];
+    e[2 * r] = x.x;
+    e[2 * r + 1] = x.y;
+  }
+  const double v0 = __ldg(a.v + elem), v1 = __ldg(a.v + elem + N), v2 = __ldg(a.v + elem + 2 * N);
+  const double* ln = a.ln + elem;
+  const double u1 = ln[LN_U1 * N], u2 = ln[LN_U2 * N];
+  const double f12 = fma(u2, v1, fma(u1, v2, ln[LN_A12 * N] * v0));
+  const double f1[3] = {v1, fma(2.0 * u1, v1, ln[LN_A11 * N] * v0), f12};
+  const double f2[3] = {v2, f12, fma(2.0 * u2, v2, ln[LN_A22 * N] * v0)};
+  const double src[3] = {0.0, fma(ln[LN_S11 * N], v1, fma(ln[LN_S12 * N], v2, ln[LN_S10 * N] * v0)),
+                         fma(ln[LN_S21 * N], v1, fma(ln[LN_S22 * N], v2, ln[LN_S20 * N] * v0))};
+#pragma unroll
+  for (int mu = 0; mu < 3; ++mu) {
+    double c = fma(dc.D[0][0], e[mu], src[mu]);
+    c = fma(dc.D[0][2], e[3 + mu], c);
+    c = fma(dc.D[0][1], f1[mu], c);
+    c = fma(dc.D[0][0], e[6 + mu], c);
+    c = fma(dc.D[0][2], e[9 + mu], c);
+    res[mu] = dscale * fma(dc.D[0][1], f2[mu], c);
+  }
+}
+
 // The imaginary half of the elements e0 .. e1 - 1 of one grid in tiles of EPB
 // elements, by a block of BLOCK >= EPB * NS^2 threads (one per solution point, the
 // rest idle), all of which call this function: share blk of nblk of the grid's
@@ -517,13 +552,14 @@ __device__ __forceinline__ void volume_tangent_range(const TanVolArgs<T>& a, con
                                                      unsigned int blk, unsigned int nblk) {
   constexpr int NN = NS * NS;
   constexpr bool F32 = sizeof(T) == 4;
+  constexpr bool NODE = !F32 && NS == 1;
   static_assert(EPB * NN <= BLOCK, "block too small for the element tile");
-  tile_dmat<T, NS, EPB, BLOCK>(a, dc, sm);
+  if constexpr (!NODE) tile_dmat<T, NS, EPB, BLOCK>(a, dc, sm);
   __shared__ double coef[MAX_NB];
   __shared__ float coef32[MAX_NB];
   if (!F32) epilogue_coefs(a.ep, coef);
   tile_coef32<T>(a.ep, coef32);
-  if (!F32)
+  if constexpr (!F32 && !NODE)
     for (int t = threadIdx.x; t < 2 * EPB; t += BLOCK) sm.sE[0][t >> 1][t & 1] = 0u;
   __syncthreads();
   const int le = threadIdx.x / NN, node = threadIdx.x % NN;
@@ -552,6 +588,13 @@ __device__ __forceinline__ void volume_tangent_range(const TanVolArgs<T>& a, con
         tile_sweep<T, NS, EPB>(a, sm, le, k1, k2, idx, Da, Db, sc, S1, S2, coef32, res);
         epilogue_node<W3, !F32>(a.ep, coef, idx, a.nodes, res, a.out, da, db, dcc, dab, dbc);
       }
+    }
+  } else if constexpr (NODE) {
+    const double dscale = -dc.two_over_dx * a.ep.scale;
+    for (long long elem = e0 + threadIdx.x; elem < e1; elem += BLOCK) {
+      double res[3];
+      volume_tangent_node(a, dc, elem, dscale, res);
+      epilogue_node<W3, true>(a.ep, coef, elem, a.nodes, res, a.out, da, db, dcc, dab, dbc);
     }
   } else {
     const double dscale = -dc.two_over_dx * a.ep.scale;

@@ -107,6 +107,7 @@ __device__ __forceinline__ double fx_ldexp(double s, int k) {
 template <int N>
 __device__ __forceinline__ double fx_dot(const double (&x)[N], const double (&wq)[N], int wexp, bool lo,
                                          const double* w0, const double* w1) {
+  if constexpr (N == 1) return (lo ? w0[0] : w1[0]) * x[0];   // one FP64 instruction either way
   unsigned m = 0u;
 #pragma unroll
   for (int k = 0; k < N; ++k) m = max(m, fx_key(x[k]));
