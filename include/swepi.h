@@ -381,7 +381,8 @@ int sw_kiops_log_clear(sw_ctx_t ctx);
  * and vector entries per orthogonalisation task.  sw_ens_tune searches them
  * per (n_e, p) class and threads per CTA in {128, 256, 512} by timing `iters`
  * batched iterations at the members' states q_dev (it overwrites the members'
- * Krylov workspace, not q).  sw_ens_set_policy: while the members that iterate
+ * Krylov workspace, not q); the untuned tiles stay where all members together
+ * run faster with them.  sw_ens_set_policy: while the members that iterate
  * hold at least theta (0..1, default 0.5) of the unfinished members' nodes, the
  * driver keeps iterating and defers the members that wait for a decision.
  * q_dev_host / stats: host arrays of `members` entries (device state vectors;
