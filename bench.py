@@ -36,8 +36,10 @@ def flops_per_jvp(ne, ns, p=4, dots=True):
     """Algorithmic FP64 flops of one Krylov JVP of the split path (the imaginary
     half of the complex-step evaluation at a fixed linearisation point; add /
     mul = 1, fma = 2) with the augmented-operator epilogue of p phi-vectors and
-    the two orthogonalisation dot products, split into the volume and face
-    kernels.  Per node: pointwise imaginary fluxes and sources 23, DFR sweeps
+    the two dot products of the new vector with the window (not the window's own
+    product, which the kernel forms beside them), split into the volume and face
+    kernels.  Most of them run as integer operations (block fixed point), so
+    their rate is no fraction of the FP64 peak.  Per node: pointwise imaginary fluxes and sources 23, DFR sweeps
     27 + 12 Ns, scaling 3, epilogue 7 p (+ 12 with the dots).  Per interface
     point: traces 12 Ns, the 3 x 6 flux map 33, hand-back 7."""
     nodes = 6 * ne * ne * ns * ns
@@ -330,16 +332,17 @@ def hbm_peak_gbs():
         return 6800.0, "fallback"
 
 
-def ortho_roofline(prof_all, wl, fused=False):
-    """The two vector passes of the window-2 orthogonalisation against HBM:
-    algorithmic bytes per Krylov iteration (orth_bytes_per_unknown) per unknown
-    of the augmented vector; the fused launch counts as the two passes."""
+def ortho_roofline(prof_all, wl, fused):
+    """The two vector passes of the window-2 orthogonalisation in one launch
+    (fused; else not reported) against HBM: algorithmic bytes per Krylov iteration
+    (orth_bytes_per_unknown) per unknown of the augmented vector; the fused launch
+    counts as the two passes."""
     o = prof_all["orthogonalisation"]
-    if not o["count"]:
+    if not o["count"] or not fused:
         return None
     pairs = o["count"] / 2.0
     t = o["ms"] * 1e-3 / pairs
-    nbytes = orth_bytes_per_unknown(2, 1, fused) * (wl.n_unknowns + 4)
+    nbytes = orth_bytes_per_unknown(2, 1, True) * (wl.n_unknowns + 4)
     peak, src = hbm_peak_gbs()
     return {"bound": "hbm", "bytes_per_iteration": nbytes, "avg_ms_per_iteration": t * 1e3,
             "achieved_gbs": nbytes / t / 1e9, "peak_gbs": peak, "frac": nbytes / t / 1e9 / peak,
@@ -360,22 +363,35 @@ def volume_bytes_per_node(ns, mode, iop, p):
     return 3 * w + 24 + window + 3 * p * w + 11 * w + 12.0 / ns * w
 
 
-def face_bytes_per_node(ns):
-    """Bytes the FP64 face kernel of a Krylov iteration must move per node: v read
-    once (24), per interface point the 18 flux-map coefficients and the three
-    fluxes handed to both sides (12 n_e^2 N_s points, 2 / N_s per node)."""
-    return 24 + (18 * 8 + 2 * 3 * 8) * 2.0 / ns
+def face_bytes_per_node(ns, mode=1):
+    """Bytes the face kernel of a Krylov iteration must move per node: v read once
+    (its FP32 copy in the complex64-bulk form), per interface point the 18 flux-map
+    coefficients and the three fluxes handed to both sides (12 n_e^2 N_s points, 2 /
+    N_s per node; FP64, or FP32 in the complex64-bulk form)."""
+    w = 8 if mode == 1 else 4
+    return 3 * w + (18 + 2 * 3) * w * 2.0 / ns
+
+
+def full_bytes_per_node(ns, kernel, iop, p):
+    """The same for the full complex-step evaluation (--jvp-mode 0): the face
+    kernel reads q and v, per interface point 12 coefficients, and hands over three
+    fluxes twice; the volume kernel reads q, v, 13 coefficients, the interface
+    fluxes, the window and the b-columns and writes Jv."""
+    if kernel == "face":
+        return 48 + (12 * 8 + 2 * 3 * 8) * 2.0 / ns
+    return 48 + 24 + 13 * 8 + 12.0 / ns * 8 + 24 * iop + 24 * p
 
 
 def orth_bytes_per_unknown(iop, mode=1, fused=False):
-    """The two vector passes of the fused window-iop orthogonalisation per unknown
-    of the augmented vector, as two launches: (read z and the iop window vectors,
-    write z) + (read z and, where the pass forms dots, iop - 1 window vectors,
-    write V_{j+1}) = 8 (2 iop + 3) B; in the complex64-bulk form the second pass
-    forms no dots and also writes the FP32 copy: 8 (iop + 2) + 20 B.  Both passes
-    in one launch (fused): each vector once, read z and the window vectors, write
-    V_{j+1} = 8 (iop + 2) B; in the complex64-bulk form the launch also forms the
-    window dots and writes the FP32 copy: 8 (iop + 2) + 4 B."""
+    """The vector passes of the window-iop orthogonalisation per unknown of the
+    augmented vector.  In one launch (fused, what the benchmark times and
+    reports): each vector once, read z and the window vectors, write V_{j+1} = 8
+    (iop + 2) B; in the complex64-bulk form the launch also forms the window dots
+    and writes the FP32 copy: 8 (iop + 2) + 4 B.  Not fused: the count of a
+    second pass that reads iop - 1 window vectors for the next dots, 8 (2 iop + 3)
+    B, in the complex64-bulk form 8 (iop + 2) + 20 B; the library's second launch
+    forms no dots any more (8 (iop + 4) B for the two), and the benchmark does not
+    report that form."""
     if fused:
         return 8.0 * (iop + 2) + (4.0 if mode == 2 else 0.0)
     if mode == 2:
@@ -383,12 +399,13 @@ def orth_bytes_per_unknown(iop, mode=1, fused=False):
     return 8.0 * (2 * iop + 3)
 
 
-def kernel_rooflines(prof, wl, mode, iop, step_ms, fp64_peak, fused=False):
+def kernel_rooflines(prof, wl, mode, iop, step_ms, fp64_peak=None, fused=False):
     """Per-kernel figures of one EPI step with every kernel family bracketed by
-    events.  FP64 kernels: algorithmic flops (flops_per_jvp, 6 more per node for
-    the third dot of window 3) against the measured FP64 peak.  HBM: the
-    algorithmic bytes (volume_bytes_per_node, orth_bytes_per_unknown) against
-    the measured copy bandwidth."""
+    events: the algorithmic bytes (volume_bytes_per_node, face_bytes_per_node,
+    orth_bytes_per_unknown) against the measured copy bandwidth, and the rate of
+    the algorithmic flops (flops_per_jvp, 6 more per node for the third dot of
+    window 3).  fp64_peak: for kernels that run those flops on the FP64 pipe, also
+    their fraction of it (the library's split kernels do not, see flops_per_jvp)."""
     hbm, _ = hbm_peak_gbs()
     nodes = 6 * wl.ne * wl.ne * wl.ns * wl.ns
     p = EPI_PHI[wl.order]
@@ -405,19 +422,20 @@ def kernel_rooflines(prof, wl, mode, iop, step_ms, fp64_peak, fused=False):
         v = {"avg_us": tv * 1e6, "launches": prof["volume_jvp"]["count"], "flops": fv,
              "bytes": vbytes, "gbs": vbytes / tv / 1e9, "hbm_frac": vbytes / tv / 1e9 / hbm}
         if mode == 1:
-            v.update({"tflops": fv / tv / 1e12, "fp64_frac": fv / tv / 1e12 / fp64_peak})
+            v["tflops"] = fv / tv / 1e12
+            if fp64_peak:
+                v["fp64_frac"] = v["tflops"] / fp64_peak
         else:
             v["fp32_tflops"] = fv / tv / 1e12
         out["volume"] = v
     if tf:
-        f = {"avg_us": tf * 1e6, "launches": prof["face_jvp"]["count"], "flops": ff}
-        if mode == 1:
-            f.update({"tflops": ff / tf / 1e12, "fp64_frac": ff / tf / 1e12 / fp64_peak})
-        else:
-            f["fp32_tflops"] = ff / tf / 1e12
+        fbytes = nodes * face_bytes_per_node(wl.ns, mode)
+        f = {"avg_us": tf * 1e6, "launches": prof["face_jvp"]["count"], "flops": ff,
+             "bytes": fbytes, "gbs": fbytes / tf / 1e9, "hbm_frac": fbytes / tf / 1e9 / hbm}
+        f["tflops" if mode == 1 else "fp32_tflops"] = ff / tf / 1e12
         out["face"] = f
     if to:
-        t = 2.0 * to   # one update-and-norm plus one scale-and-dot pass per Krylov iteration
+        t = 2.0 * to   # the update and the scaling of a Krylov iteration count as two passes, in one launch or two
         obytes = orth_bytes_per_unknown(iop, mode, fused) * (wl.n_unknowns + 4)
         out["orthogonalisation"] = {"avg_us_per_iteration": t * 1e6, "bytes_per_iteration": obytes,
                                     "gbs": obytes / t / 1e9, "hbm_frac": obytes / t / 1e9 / hbm}
@@ -425,17 +443,17 @@ def kernel_rooflines(prof, wl, mode, iop, step_ms, fp64_peak, fused=False):
         out["expm"] = {"avg_us": avg("expm") * 1e6, "launches": prof["expm"]["count"]}
     out["share_of_step"] = {k: prof[k]["ms"] / step_ms
                             for k in ("volume_jvp", "face_jvp", "orthogonalisation", "expm", "linearize")}
-    out["peaks"] = {"fp64_tflops": fp64_peak, "hbm_gbs": hbm}
+    out["peaks"] = {"hbm_gbs": hbm}
     return out
 
 
 def fp32_form_comparison(args, dev, workload="ne30_p5", variants=(("fp64", 1, 2), ("complex64_bulk", 2, 2)),
-                         fp64_peak=None, total_steps=None, dt=None):
+                         per_kernel=False, total_steps=None, dt=None):
     """The complex64-bulk form against the FP64 path: steps/s of each variant
     (name, JVP mode, orthogonalisation window[, "learned": the learned initial
     substep after the warm-up]) from the same start, each variant's state
     difference to the first (the FP64 path, window 2) after the run, and the EPI
-    time-discretisation error (FP64 at dt against dt/4).  With fp64_peak, each
+    time-discretisation error (FP64 at dt against dt/4).  With per_kernel, each
     variant then takes one more step with every kernel family bracketed by
     events (after its state was kept) and reports per-kernel rooflines."""
     import torch
@@ -463,8 +481,9 @@ def fp32_form_comparison(args, dev, workload="ne30_p5", variants=(("fp64", 1, 2)
         ctx.set_jvp_mode(mode)
         if extra == "device":   # the phi-function solver's controller on the device (one CUDA graph per call)
             ctx.set_kiops_driver(1)
-        # both vector passes in one launch (the host controller; the device graph keeps two)
-        fused = bool(ctx.set_orth_fused(1)) and extra != "device"
+        # both vector passes in one launch (the device controller's graph keeps two, but a profiled step runs the
+        # host controller)
+        fused = bool(ctx.set_orth_fused(1))
         h0max = float(q.view(3, -1)[0].abs().max())
         done = 0   # EPI steps completed (reported with a failure)
         try:
@@ -487,7 +506,7 @@ def fp32_form_comparison(args, dev, workload="ne30_p5", variants=(("fp64", 1, 2)
             res[name] = timed * mult / (e0.elapsed_time(e1) * 1e-3)
             stats[name] = kry / (timed * mult)
             states[name] = q.view(3, -1).clone()
-            if fp64_peak is not None and mult == 1:
+            if per_kernel and mult == 1:
                 try:   # a failure here leaves the variant's timing and state in place
                     ctx.profile(True)
                     b0 = torch.cuda.Event(enable_timing=True)
@@ -497,7 +516,9 @@ def fp32_form_comparison(args, dev, workload="ne30_p5", variants=(("fp64", 1, 2)
                     b1.record()
                     torch.cuda.synchronize()
                     kernels[name] = kernel_rooflines(ctx.profile_read(), wl, mode, iop, b0.elapsed_time(b1),
-                                                     fp64_peak, fused)
+                                                     fused=fused)
+                    if not fused:
+                        kernels[name].pop("orthogonalisation", None)
                 except Exception as e:
                     kernels[name] = {"error": f"{type(e).__name__}: {e}"[:200]}
                 ctx.profile(False)
@@ -552,7 +573,7 @@ ORACLE_STEP_NE60_P5 = {"krylov_iters": 384, "attempts": 13, "substeps": 3, "seco
                        "host": "one x86-64 core of the build container (the counts do not depend on the host)"}
 
 
-def ensemble_form(args, dev, fp64_peak):
+def ensemble_form(args, dev):
     """The batched ensemble: 96 members on uneven grids (n_e in {8, 16, 24, 32},
     p in {3, 4, 5}, EPI4/5, dt = 900 s, degree <= 12 perturbations of 50 m)
     for 24 steps through sw_ens_epi_run after autotuning; against one member
@@ -598,11 +619,13 @@ def ensemble_form(args, dev, fp64_peak):
     for i, r in zip(idx, refs):
         a, b = ys[i].view(3, -1), r.view(3, -1)
         diff = max(diff, max(float(torch.linalg.norm(a[k] - b[k]) / torch.linalg.norm(b[k])) for k in range(3)))
-    fl = 0.0
+    fl = nb = 0.0
     for m, k in zip(members, krylov):
-        fv, ff = flops_per_jvp(m.ne, m.ns, p=m.order - 1)
-        fl += k * (fv + ff)
-    achieved = fl / (info["iter_ms"] * 1e-3) / 1e12 if info["iter_ms"] > 0 else None
+        fl += k * sum(flops_per_jvp(m.ne, m.ns, p=m.order - 1))
+        # the update task reads z and two window vectors and writes z, the scaling reads and writes it: 48 B
+        nb += k * m.nodes * (volume_bytes_per_node(m.ns, 1, 2, EPI_PHI[m.order]) + face_bytes_per_node(m.ns) + 3 * 48)
+    iter_s = info["iter_ms"] * 1e-3
+    hbm, _ = hbm_peak_gbs()
     return {"members": len(members), "steps": steps, "seconds": sec,
             "members_per_s": len(members) / sec, "member_steps_per_s": len(members) * steps / sec,
             "jvp_dof_per_s": sum(k * 3 * m.nodes for m, k in zip(members, krylov)) / sec,
@@ -612,8 +635,9 @@ def ensemble_form(args, dev, fp64_peak):
             "gpu_launches": info["launches"], "block": info["block"], "ctas": info["ctas"],
             "tiles_by_class": tiles,
             "iteration_kernel": {"ms": info["iter_ms"], "share_of_run": info["iter_ms"] * 1e-3 / sec,
-                                 "fp64_tflops": achieved, "peak_tflops": fp64_peak,
-                                 "frac": (achieved / fp64_peak) if achieved and fp64_peak else None},
+                                 "tflops": fl / iter_s / 1e12 if iter_s > 0 else None, "bytes": nb,
+                                 "gbs": nb / iter_s / 1e9 if iter_s > 0 else None,
+                                 "hbm_frac": nb / iter_s / 1e9 / hbm if iter_s > 0 else None},
             "single_member_path": {"members": len(idx), "seconds": single_s,
                                    "member_steps_per_s": len(idx) * steps / single_s},
             "max_rel_l2_vs_single": diff, "members_with_equal_krylov_count": same_krylov, "build_s": build_s}
@@ -864,24 +888,20 @@ def main():
         vj, fj = prof["volume_jvp"], prof_all["face_jvp"]
         t_vol = vj["ms"] / max(1, vj["count"]) * 1e-3
         t_face = fj["ms"] / max(1, fj["count"]) * 1e-3
-        peak = swepi.sw_fp64_fma_peak()
         dominant = "volume" if prof_all["volume_jvp"]["ms"] >= prof_all["face_jvp"]["ms"] else "face"
-        if args.jvp_mode == 1:
-            # the split kernels do most of their arithmetic in block fixed point on the integer pipe, so
-            # the FP64 peak is no roofline of theirs: the bytes they must move are
-            rpeak, peak_src = hbm_peak_gbs()
-            nodes = 6 * ne * ne * ns * ns
-            if dominant == "volume":
-                bound, nb = "hbm", nodes * volume_bytes_per_node(ns, 1, 2, EPI_PHI[wl.order])
-            else:
-                bound, nb = "hbm", face_bytes_per_node(ns) * nodes
-            achieved, unit = nb / (t_vol if dominant == "volume" else t_face) / 1e9, "GB/s"
-            peak_src = f"HBM copy bandwidth ({peak_src}); algorithmic bytes {nb:.4g} a launch"
+        # these kernels do most of their arithmetic in block fixed point on the integer pipe, so the FP64 peak is
+        # no roofline of theirs: the bytes they must move are
+        rpeak, peak_src = hbm_peak_gbs()
+        nodes = 6 * ne * ne * ns * ns
+        if args.jvp_mode == 0:
+            nb = nodes * full_bytes_per_node(ns, dominant, 2, EPI_PHI[wl.order])
+        elif dominant == "volume":
+            nb = nodes * volume_bytes_per_node(ns, 1, 2, EPI_PHI[wl.order])
         else:
-            bound, unit, rpeak = "alu", "TFLOP/s", peak
-            peak_src = "FP64 FMA throughput measured live by sw_fp64_fma_peak (nominal 1.25)"
-            achieved = (fv / t_vol if dominant == "volume" else ff / t_face) / 1e12
-        roofline = {"bound": bound, "achieved": achieved, "peak": rpeak, "unit": unit,
+            nb = nodes * face_bytes_per_node(ns)
+        achieved = nb / (t_vol if dominant == "volume" else t_face) / 1e9
+        peak_src = f"HBM copy bandwidth ({peak_src}); algorithmic bytes {nb:.4g} a launch"
+        roofline = {"bound": "hbm", "achieved": achieved, "peak": rpeak, "unit": "GB/s",
                     "frac": achieved / rpeak,
                     "traffic": TRAFFIC_BYTES.get(wl.name) if dominant == "volume" and args.jvp_mode == 1 else None,
                     "kernel": ((f"volume_tangent_kernel<double,{ns}>" if dominant == "volume"
@@ -956,16 +976,16 @@ def main():
                                            ("complex64_bulk_window3_learned", 2, 3, "learned"),
                                            ("fp64_device_controller", 1, 2, "device"),
                                            ("complex64_bulk_window3_device_controller", 2, 3, "device")),
-                    fp64_peak=peak, total_steps=48))
+                    per_kernel=True, total_steps=48))
             if world == 1 and not args.no_ensemble:
-                form("ensemble_96", lambda: ensemble_form(args, dev, peak))
+                form("ensemble_96", lambda: ensemble_form(args, dev))
             if world == 1 and not args.no_large:
                 # the large single instance: 6 x 90 x 90 elements, p = 6, bottom topography, EPI6 over its
                 # configured 36 steps at dt = 600 s: at the configured 1200 s (and at 900 s) the FP64 method
                 # itself goes unstable within the 36 steps (the order-6 vorticity growth), at 600 s both
                 # forms stay finite
                 form("large_ne90_p6", lambda: fp32_form_comparison(
-                    args, dev, "ne90_p6", (("fp64", 1, 2), ("complex64_bulk_window3", 2, 3)), fp64_peak=peak,
+                    args, dev, "ne90_p6", (("fp64", 1, 2), ("complex64_bulk_window3", 2, 3)), per_kernel=True,
                     total_steps=36, dt=LARGE_STABLE_DT))
         if world == 1 and not args.no_cpu_baseline:
             counts = (krylov / args.steps, attempts / args.steps, substeps / args.steps)
