@@ -210,8 +210,12 @@ def _dev_ptr(t, n=None):
 def _stream(stream):
     if stream is not None:
         return ctypes.c_void_p(stream.cuda_stream)
-    torch = _torch()   # the current stream's handle, without a Stream object around it
-    return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+    torch = _torch()
+    # the current stream's handle, without a Stream object around it where this PyTorch has the (private) call
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return ctypes.c_void_p(raw(torch.cuda.current_device()))
 
 
 def _host(a, n):
