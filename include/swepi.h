@@ -474,7 +474,8 @@ int sw_check_status(int* checked);
  * context's device table, so that the next face kernel's check fires (the
  * test of the checks); what = 0 moves it back; what = 2 leaves counts in the
  * phi-function solver's tickets, as a call whose bounded wait gave up can
- * (SW_EINVAL before the context's first such call). */
+ * (SW_EINVAL while the context has none: before its first phi-function call or
+ * complex64-bulk linearisation). */
 int sw_check_inject(sw_ctx_t ctx, int what);
 
 /* Measured FP64 fused-multiply-add throughput of the current device in

@@ -407,6 +407,7 @@ int launch_linearize(Ctx& c, const double* q, cudaStream_t s) {
     if (!c.d_lin_face32 && cudaMalloc(&c.d_lin_face32, sizeof(float) * 23 * c.nfacepts) != cudaSuccess)
       return SW_ENOMEM;
     if (!c.d_v32 && cudaMalloc(&c.d_v32, sizeof(float) * c.n) != cudaSuccess) return SW_ENOMEM;
+    if (int rc = ensure_flags(c)) return rc;   // where the staged kernel's bounded waits report
   }
   if (!c.d_lin_face && cudaMalloc(&c.d_lin_face, sizeof(double) * 18 * c.nfacepts) != cudaSuccess)
     return SW_ENOMEM;

@@ -57,6 +57,12 @@ void free_ptr(double*& p) {
 }
 }  // namespace
 
+int ensure_flags(Ctx& c) {
+  if (c.d_flags) return SW_OK;
+  if (cudaMalloc(&c.d_flags, sizeof(int) * 16) != cudaSuccess) return SW_ENOMEM;
+  return cuda_status(cudaMemset(c.d_flags, 0, sizeof(int) * 16));
+}
+
 int ensure_krylov(Ctx& c, int m_max) {
   if (c.vcap >= m_max + 1 && c.d_V) return SW_OK;
   free_ptr(c.d_V);
@@ -77,10 +83,7 @@ int ensure_krylov(Ctx& c, int m_max) {
   free_ptr(c.d_cdot);
   if (cudaMalloc(&c.d_cdot, sizeof(double) * c.ldh) != cudaSuccess) return SW_ENOMEM;
   if (!c.d_scal && cudaMalloc(&c.d_scal, sizeof(double) * 64) != cudaSuccess) return SW_ENOMEM;
-  if (!c.d_flags) {
-    if (cudaMalloc(&c.d_flags, sizeof(int) * 16) != cudaSuccess) return SW_ENOMEM;
-    if (cudaMemset(c.d_flags, 0, sizeof(int) * 16) != cudaSuccess) return SW_ECUDA;
-  }
+  if (int rc = ensure_flags(c)) return rc;
   if (!c.h_pinned && cudaMallocHost(&c.h_pinned, sizeof(double) * 64) != cudaSuccess) return SW_ENOMEM;
   if (cudaMemset(c.d_V, 0, sizeof(double) * c.ldv * c.vcap) != cudaSuccess) return SW_ECUDA;
   return SW_OK;

@@ -353,6 +353,7 @@ int launch_lincomb(Ctx& c, double* out, long long n, int k, const double* const*
 int kiops_run(Ctx& c, const double* q_lin, double dt, double tau_out, int nb, const double* const* b,
               const sw_kiops_opts& o, double* w, sw_kiops_stats* st, cudaStream_t s, bool use_lin);
 int ensure_krylov(Ctx& c, int m_max);
+int ensure_flags(Ctx& c);
 // before a call's first reduction: the gave-up mark, the tickets and the barrier
 // counter, which a call whose bounded wait gave up leaves mid-count (a reduction
 // that starts from such a count never publishes its sum, or does so too early)

@@ -47,6 +47,13 @@ for driver in (0, 1):
         assert res[0][1] == res[1][1], (driver, mode, res[0][1], res[1][1])
         assert torch.equal(res[0][0], res[1][0]), (driver, mode)
 
+# the complex64-bulk product alone: its bounded waits have a place to report to from the linearisation on
+ctx = swepi.SWContext(g.ne, g.ns - 1, g.rotation)
+ctx.set_jvp_mode(2)
+ctx.linearize(qd)
+swepi.sw_check_inject(ctx.handle, 2)   # refused while the context has no flags
+assert torch.isfinite(ctx.jvp_linearized(b[1])).all()
+
 res = []
 for planted in (False, True):
     ctxs = [context(0, 1) for _ in range(2)]
