@@ -43,15 +43,5 @@ __device__ __forceinline__ double f32_to_f64_bits(float f) {
   hi = (e == 255u) ? (sign | 0x7ff00000u | (m >> 3) | (m ? 0x80000u : 0u)) : hi;
   return __hiloint2double((int)hi, (int)lo);
 }
-template <typename T>
-__device__ __forceinline__ T from_f64(double x) {
-  if constexpr (sizeof(T) == 4) return f64_to_f32_bits(x);
-  else return x;
-}
-template <typename T>
-__device__ __forceinline__ double to_f64(T x) {
-  if constexpr (sizeof(T) == 4) return f32_to_f64_bits(x);
-  else return x;
-}
 
 }  // namespace swepi

@@ -353,6 +353,12 @@ __device__ __forceinline__ void block_sums(double v[K], double* sbuf) {
   }
 }
 
+// the shift of the augmented tail (block 0)
+__device__ __forceinline__ void epilogue_tail(const AugEpilogue& ep, unsigned int blk) {
+  if (ep.tail_out && blk == 0 && threadIdx.x < ep.p)
+    ep.tail_out[threadIdx.x] = (threadIdx.x + 1 < ep.p) ? ep.tail_in[threadIdx.x + 1] : 0.0;
+}
+
 // Second half of the volume epilogue (all threads of the block call it, with
 // their partial sums over their nodes, see epilogue_node): the shift of the
 // augmented tail, the tail's share of the dots, the block sums and -- in the
@@ -362,8 +368,7 @@ template <int THREADS, bool W3>
 __device__ __forceinline__ void epilogue_finish(const AugEpilogue& ep, double da, double db, double dcc,
                                                 unsigned int blk, unsigned int nblk, double dab, double dbc,
                                                 double* sbuf) {
-  if (ep.tail_out && blk == 0 && threadIdx.x < ep.p)
-    ep.tail_out[threadIdx.x] = (threadIdx.x + 1 < ep.p) ? ep.tail_in[threadIdx.x + 1] : 0.0;
+  epilogue_tail(ep, blk);
   if (!ep.dotB) return;   // uniform over the grid
   if (blk == 0 && threadIdx.x == 0) {
     for (int l = 0; l < ep.p; ++l) {

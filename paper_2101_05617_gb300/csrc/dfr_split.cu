@@ -274,9 +274,14 @@ int linearize_ns(Ctx& c, const double* q, cudaStream_t s) {
   return cuda_status(cudaGetLastError());
 }
 
+// the complex64-bulk form's orthogonalisation dots are a pass of their own
+template <typename T>
+constexpr bool kDots = sizeof(T) == 8;
+
 template <typename T, int NS>
 int tangent_ns(Ctx& c, const double* v, double* out, const AugEpilogue& ep, const T* ln, const T* lf, T* fb,
                cudaStream_t s) {
+  if (!kDots<T> && ep.dotB) return SW_EINVAL;
   const bool pf = prof_take(c, PK_FACE_JVP), pv = prof_take(c, PK_VOL_JVP);
   cudaEvent_t e0 = nullptr, e1 = nullptr, e2 = nullptr;
   if (pf) {
@@ -301,14 +306,18 @@ int tangent_ns(Ctx& c, const double* v, double* out, const AugEpilogue& ep, cons
     if (rt == SW_OK) c.launches--;   // counted below
   }
   if (rt != SW_OK) {
-    const int ctas = ep.dotC ? volume_ctas<T, NS, true, false>(c.device, vblocks)
-                             : volume_ctas<T, NS, false, false>(c.device, vblocks);
-    if (ctas < 1) return SW_ECUDA;
-    const cudaError_t ev = ep.dotC ? launch_pdl(volume_tangent_kernel<T, NS, true>, dim3((unsigned)ctas),
-                                                 dim3(VolShape<NS>::THREADS), s, va, c.dc)
-                                   : launch_pdl(volume_tangent_kernel<T, NS, false>, dim3((unsigned)ctas),
-                                                dim3(VolShape<NS>::THREADS), s, va, c.dc);
-    if (ev != cudaSuccess) return SW_ECUDA;
+    auto launch = [&](auto kernel, int ctas) {
+      if (ctas < 1) return false;
+      return launch_pdl(kernel, dim3((unsigned)ctas), dim3(VolShape<NS>::THREADS), s, va, c.dc) == cudaSuccess;
+    };
+    bool ok;
+    if constexpr (kDots<T>) {
+      ok = ep.dotC ? launch(volume_tangent_kernel<T, NS, true>, volume_ctas<T, NS, true, false>(c.device, vblocks))
+                   : launch(volume_tangent_kernel<T, NS, false>, volume_ctas<T, NS, false, false>(c.device, vblocks));
+    } else {
+      ok = launch(volume_tangent_kernel<T, NS, false>, volume_ctas<T, NS, false, false>(c.device, vblocks));
+    }
+    if (!ok) return SW_ECUDA;
   }
   if (pv) {
     e2 = prof_event(c);
@@ -338,18 +347,23 @@ int capture_iter_ns(Ctx& c, KDev* kd, const KFix& f, bool w3, int p, cudaStream_
   c.launches++;
   if (cudaGetLastError() != cudaSuccess) return SW_ECUDA;
   if (fp32 && p <= kTileMaxB) {   // the staged kernel where the buffers allow it
-    const int rt = capture_volume_tile_dev<NS>(c, kd, f, w3, s);
+    const int rt = capture_volume_tile_dev<NS>(c, kd, f, s);
     if (rt <= 0) return rt;
   }
   TanVolArgs<T> va{nullptr, c.nodes, c.nelem, ln, c.d_lin_exp, fb, nullptr, AugEpilogue{}};
   const long long vblocks = (c.nelem + VolShape<NS>::EPB - 1) / VolShape<NS>::EPB;
-  const int ctas = w3 ? volume_ctas<T, NS, true, true>(c.device, vblocks)
-                      : volume_ctas<T, NS, false, true>(c.device, vblocks);
-  if (ctas < 1) return SW_ECUDA;
-  if (w3)
-    volume_tangent_dev_kernel<T, NS, true><<<(unsigned)ctas, VolShape<NS>::THREADS, 0, s>>>(kd, f, va, c.dc);
-  else
-    volume_tangent_dev_kernel<T, NS, false><<<(unsigned)ctas, VolShape<NS>::THREADS, 0, s>>>(kd, f, va, c.dc);
+  auto launch = [&](auto kernel, int ctas) {
+    if (ctas > 0) kernel<<<(unsigned)ctas, VolShape<NS>::THREADS, 0, s>>>(kd, f, va, c.dc);
+    return ctas > 0;
+  };
+  bool ok;
+  if constexpr (kDots<T>) {
+    ok = w3 ? launch(volume_tangent_dev_kernel<T, NS, true>, volume_ctas<T, NS, true, true>(c.device, vblocks))
+            : launch(volume_tangent_dev_kernel<T, NS, false>, volume_ctas<T, NS, false, true>(c.device, vblocks));
+  } else {
+    ok = launch(volume_tangent_dev_kernel<T, NS, false>, volume_ctas<T, NS, false, true>(c.device, vblocks));
+  }
+  if (!ok) return SW_ECUDA;
   c.launches++;
   return cuda_status(cudaGetLastError());
 }
@@ -362,7 +376,7 @@ int capture_iter_any(Ctx& c, KDev* kd, const KFix& f, bool fp32, bool w3, int p,
 template <int NS>
 int prepare_dev_ns(const Ctx& c, bool fp32) {
   const int a = fp32 ? volume_ctas<float, NS, false, true>(c.device, 1) : volume_ctas<double, NS, false, true>(c.device, 1);
-  const int b = fp32 ? volume_ctas<float, NS, true, true>(c.device, 1) : volume_ctas<double, NS, true, true>(c.device, 1);
+  const int b = fp32 ? a : volume_ctas<double, NS, true, true>(c.device, 1);
   return (a < 1 || b < 1) ? SW_ECUDA : SW_OK;
 }
 

@@ -129,7 +129,8 @@ struct VolSmem {
   T sF[EPB][2][3][NS * NS];   // fluxes along xi^1 and xi^2
   T sB[EPB][4][3][NS];        // interface fluxes of the four edges
   T sD[NS][NS + 3];           // derivative matrix, padded rows: distinct banks per k
-  unsigned sE[2][EPB][2];     // FP64: largest magnitude keys of the elements' fluxes (mass, momentum), by tile parity
+  // FP64: largest magnitude keys of the elements' fluxes (mass, momentum), by tile parity
+  unsigned sE[sizeof(T) == 8 ? 2 : 1][sizeof(T) == 8 ? EPB : 1][2];
 };
 
 // derivative matrix into shared memory: in FP32 pre-multiplied by -(2/dx) *
@@ -140,38 +141,39 @@ template <typename T, int NS, int EPB, int BLOCK>
 __device__ __forceinline__ void tile_dmat(const TanVolArgs<T>& a, const DfrConst& dc, VolSmem<T, NS, EPB>& sm) {
   const double dscale = -dc.two_over_dx * a.ep.scale;
   for (int t = threadIdx.x; t < NS * (NS + 2); t += BLOCK) {
-    if constexpr (sizeof(T) == 4) sm.sD[t / (NS + 2)][t % (NS + 2)] = from_f64<T>(dscale * dc.D[t / (NS + 2)][t % (NS + 2)]);
+    if constexpr (sizeof(T) == 4) sm.sD[t / (NS + 2)][t % (NS + 2)] = f64_to_f32_bits(dscale * dc.D[t / (NS + 2)][t % (NS + 2)]);
     else sm.sD[t / (NS + 2)][t % (NS + 2)] = dc.Dq[t / (NS + 2)][t % (NS + 2)];
   }
 }
 
+// ---- FP32 (complex64-bulk form)
 // interface fluxes of the four edges of the elements eb .. eb + EPB - 1 (those
 // below e_end) into shared memory
-template <typename T, int NS, int EPB, int BLOCK>
-__device__ __forceinline__ void tile_edges(const TanVolArgs<T>& a, VolSmem<T, NS, EPB>& sm, long long eb,
+template <int NS, int EPB, int BLOCK>
+__device__ __forceinline__ void tile_edges(const TanVolArgs<float>& a, VolSmem<float, NS, EPB>& sm, long long eb,
                                            long long e_end) {
   for (int t = threadIdx.x; t < EPB * 12 * NS; t += BLOCK) {
     const int e = t / (12 * NS), r = t % (12 * NS);
     const long long ge = eb + e;
-    (&sm.sB[e][0][0][0])[r] = (ge < e_end) ? a.fb[ge * 12 * NS + r] : T(0);
+    (&sm.sB[e][0][0][0])[r] = (ge < e_end) ? a.fb[ge * 12 * NS + r] : 0.f;
   }
 }
 
 // pointwise imaginary fluxes of node idx (element le of the tile, node
 // `node`) into shared memory; the sources S^1, S^2 returned
-template <typename T, int NS, int EPB>
-__device__ __forceinline__ void tile_fluxes(const TanVolArgs<T>& a, VolSmem<T, NS, EPB>& sm, int le, int node,
-                                            long long idx, T& S1, T& S2) {
+template <int NS, int EPB>
+__device__ __forceinline__ void tile_fluxes(const TanVolArgs<float>& a, VolSmem<float, NS, EPB>& sm, int le, int node,
+                                            long long idx, float& S1, float& S2) {
   const long long N = a.nodes;
-  const T v0 = from_f64<T>(__ldg(a.v + idx)), v1 = from_f64<T>(__ldg(a.v + idx + N));
-  const T v2 = from_f64<T>(__ldg(a.v + idx + 2 * N));
-  const T* ln = a.ln + idx;
-  const T u1 = ln[LN_U1 * N], u2 = ln[LN_U2 * N];
-  const T F11 = fma(T(2) * u1, v1, ln[LN_A11 * N] * v0);
-  const T F12 = fma(u2, v1, fma(u1, v2, ln[LN_A12 * N] * v0));
-  const T F22 = fma(T(2) * u2, v2, ln[LN_A22 * N] * v0);
-  S1 = fma(ln[LN_S11 * N], v1, fma(ln[LN_S12 * N], v2, ln[LN_S10 * N] * v0));
-  S2 = fma(ln[LN_S21 * N], v1, fma(ln[LN_S22 * N], v2, ln[LN_S20 * N] * v0));
+  const float v0 = f64_to_f32_bits(__ldg(a.v + idx)), v1 = f64_to_f32_bits(__ldg(a.v + idx + N));
+  const float v2 = f64_to_f32_bits(__ldg(a.v + idx + 2 * N));
+  const float* ln = a.ln + idx;
+  const float u1 = ln[LN_U1 * N], u2 = ln[LN_U2 * N];
+  const float F11 = fmaf(2.f * u1, v1, ln[LN_A11 * N] * v0);
+  const float F12 = fmaf(u2, v1, fmaf(u1, v2, ln[LN_A12 * N] * v0));
+  const float F22 = fmaf(2.f * u2, v2, ln[LN_A22 * N] * v0);
+  S1 = fmaf(ln[LN_S11 * N], v1, fmaf(ln[LN_S12 * N], v2, ln[LN_S10 * N] * v0));
+  S2 = fmaf(ln[LN_S21 * N], v1, fmaf(ln[LN_S22 * N], v2, ln[LN_S20 * N] * v0));
   sm.sF[le][0][0][node] = v1;
   sm.sF[le][0][1][node] = F11;
   sm.sF[le][0][2][node] = F12;
@@ -460,47 +462,44 @@ __device__ __forceinline__ void tan_sweep(const double (*sF)[3][NS * NS], const 
   fx_sweep<NS, false>(sF, sB, k1, k2, Da, Db, dc, dscale, fixed, fx_exp(M0), TF, s1, s2, add1, add2, res);
 }
 
-// the two DFR sweeps of one node (rows Da, Db of the scaled derivative
-// matrix) started from sc * source; in the complex64-bulk form also the
-// b-column terms nu y_l b_l in FP32 (coef32: the rounded nu y_l)
-template <typename T, int NS, int EPB>
-__device__ __forceinline__ void tile_sweep(const TanVolArgs<T>& a, const VolSmem<T, NS, EPB>& sm, int le, int k1,
-                                           int k2, long long idx, const T (&Da)[NS + 2], const T (&Db)[NS + 2],
-                                           T sc, T S1, T S2, const float* coef32, double res[3]) {
-  const T src[3] = {T(0), S1, S2};
-  T acc[3];
+// FP32: the two DFR sweeps of one node (rows Da, Db of the scaled derivative
+// matrix) started from sc * source, and the b-column terms nu y_l b_l (coef32: the
+// rounded nu y_l)
+template <int NS, int EPB>
+__device__ __forceinline__ void tile_sweep(const TanVolArgs<float>& a, const VolSmem<float, NS, EPB>& sm, int le, int k1,
+                                           int k2, long long idx, const float (&Da)[NS + 2], const float (&Db)[NS + 2],
+                                           float sc, float S1, float S2, const float* coef32, double res[3]) {
+  const float src[3] = {0.f, S1, S2};
+  float acc[3];
 #pragma unroll
   for (int mu = 0; mu < 3; ++mu) {
-    T c = (mu == 0) ? T(0) : sc * src[mu];
-    c = fma(Da[0], sm.sB[le][0][mu][k2], c);
-    c = fma(Da[NS + 1], sm.sB[le][1][mu][k2], c);
+    float c = (mu == 0) ? 0.f : sc * src[mu];
+    c = fmaf(Da[0], sm.sB[le][0][mu][k2], c);
+    c = fmaf(Da[NS + 1], sm.sB[le][1][mu][k2], c);
 #pragma unroll
-    for (int l = 0; l < NS; ++l) c = fma(Da[l + 1], sm.sF[le][0][mu][k2 * NS + l], c);
-    c = fma(Db[0], sm.sB[le][2][mu][k1], c);
-    c = fma(Db[NS + 1], sm.sB[le][3][mu][k1], c);
+    for (int l = 0; l < NS; ++l) c = fmaf(Da[l + 1], sm.sF[le][0][mu][k2 * NS + l], c);
+    c = fmaf(Db[0], sm.sB[le][2][mu][k1], c);
+    c = fmaf(Db[NS + 1], sm.sB[le][3][mu][k1], c);
 #pragma unroll
-    for (int l = 0; l < NS; ++l) c = fma(Db[l + 1], sm.sF[le][1][mu][l * NS + k1], c);
+    for (int l = 0; l < NS; ++l) c = fmaf(Db[l + 1], sm.sF[le][1][mu][l * NS + k1], c);
     acc[mu] = c;
   }
-  if constexpr (sizeof(T) == 4) {
-    const long long N = a.nodes;
-    const int p = a.ep.p < MAX_NB ? a.ep.p : MAX_NB;
+  const long long N = a.nodes;
+  const int p = a.ep.p < MAX_NB ? a.ep.p : MAX_NB;
 #pragma unroll 1
-    for (int l = 0; l < p; ++l) {
-      const float* bl = a.ep.b32[l];
-      if (!bl) continue;
+  for (int l = 0; l < p; ++l) {
+    const float* bl = a.ep.b32[l];
+    if (!bl) continue;
 #pragma unroll
-      for (int mu = 0; mu < 3; ++mu) acc[mu] = fma(T(coef32[l]), T(__ldg(bl + idx + mu * N)), acc[mu]);
-    }
+    for (int mu = 0; mu < 3; ++mu) acc[mu] = fmaf(coef32[l], __ldg(bl + idx + mu * N), acc[mu]);
   }
 #pragma unroll
-  for (int mu = 0; mu < 3; ++mu) res[mu] = to_f64<T>(acc[mu]);
+  for (int mu = 0; mu < 3; ++mu) res[mu] = f32_to_f64_bits(acc[mu]);
 }
 
 // the complex64-bulk form's FP32 tail coefficients nu * y_l (once per block)
-template <typename T>
 __device__ __forceinline__ void tile_coef32(const AugEpilogue& ep, float* coef32) {
-  if (sizeof(T) == 4 && threadIdx.x < MAX_NB) {
+  if (threadIdx.x < MAX_NB) {
     const int l = threadIdx.x;
     coef32[l] = (l < ep.p && ep.b32[l]) ? f64_to_f32_bits(ep.tail_in[l]) : 0.f;
   }
@@ -558,7 +557,7 @@ __device__ __forceinline__ void volume_tangent_range(const TanVolArgs<T>& a, con
   __shared__ double coef[MAX_NB];
   __shared__ float coef32[MAX_NB];
   if (!F32) epilogue_coefs(a.ep, coef);
-  tile_coef32<T>(a.ep, coef32);
+  if constexpr (F32) tile_coef32(a.ep, coef32);
   if constexpr (!F32 && !NODE)
     for (int t = threadIdx.x; t < 2 * EPB; t += BLOCK) sm.sE[0][t >> 1][t & 1] = 0u;
   __syncthreads();
@@ -573,19 +572,19 @@ __device__ __forceinline__ void volume_tangent_range(const TanVolArgs<T>& a, con
       Da[n] = lane_on ? sm.sD[k1][n] : T(0);
       Db[n] = lane_on ? sm.sD[k2][n] : T(0);
     }
-    const T sc = from_f64<T>(a.ep.scale);
+    const float sc = f64_to_f32_bits(a.ep.scale);
     for (long long eb = e0; eb < e1; eb += EPB) {
       const long long elem = eb + le;
       const bool active = lane_on && elem < e1;
       const long long idx = elem * NN + node;
       __syncthreads();   // the previous tile's readers are done with sF and sB
-      tile_edges<T, NS, EPB, BLOCK>(a, sm, eb, e1);
+      tile_edges<NS, EPB, BLOCK>(a, sm, eb, e1);
       T S1 = T(0), S2 = T(0);
-      if (active) tile_fluxes<T, NS, EPB>(a, sm, le, node, idx, S1, S2);
+      if (active) tile_fluxes<NS, EPB>(a, sm, le, node, idx, S1, S2);
       __syncthreads();
       if (active) {
         double res[3];
-        tile_sweep<T, NS, EPB>(a, sm, le, k1, k2, idx, Da, Db, sc, S1, S2, coef32, res);
+        tile_sweep<NS, EPB>(a, sm, le, k1, k2, idx, Da, Db, sc, S1, S2, coef32, res);
         epilogue_node<W3, !F32>(a.ep, coef, idx, a.nodes, res, a.out, da, db, dcc, dab, dbc);
       }
     }

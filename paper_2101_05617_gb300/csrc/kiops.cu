@@ -78,7 +78,7 @@ int ensure_krylov(Ctx& c, int m_max) {
   if (cudaMalloc(&c.d_H, sizeof(double) * c.ldh * c.ldh) != cudaSuccess) return SW_ENOMEM;
   if (cudaMalloc(&c.d_F, sizeof(double) * c.ldh * c.ldh) != cudaSuccess) return SW_ENOMEM;
   if (cudaMalloc(&c.d_expm_ws, sizeof(double) * 8 * 160 * 160) != cudaSuccess) return SW_ENOMEM;
-  if (!c.d_partials && cudaMalloc(&c.d_partials, sizeof(double) * 6 * RED_BLOCKS) != cudaSuccess) return SW_ENOMEM;
+  if (!c.d_partials && cudaMalloc(&c.d_partials, sizeof(double) * 5 * RED_BLOCKS) != cudaSuccess) return SW_ENOMEM;
   if (!c.d_vpart && cudaMalloc(&c.d_vpart, sizeof(double) * 5 * (c.nelem + 1)) != cudaSuccess) return SW_ENOMEM;
   free_ptr(c.d_cdot);
   if (cudaMalloc(&c.d_cdot, sizeof(double) * c.ldh) != cudaSuccess) return SW_ENOMEM;

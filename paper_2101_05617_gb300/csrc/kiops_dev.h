@@ -85,7 +85,7 @@ int capture_iter_jvp(Ctx& c, KDev* kd, const KFix& f, bool fp32, bool w3, int p,
 // the staged complex64-bulk volume kernel in that form (dfr_tile.cu); 1 when
 // the context's buffers are not eligible
 template <int NS>
-int capture_volume_tile_dev(Ctx& c, KDev* kd, const KFix& f, bool w3, cudaStream_t s);
+int capture_volume_tile_dev(Ctx& c, KDev* kd, const KFix& f, cudaStream_t s);
 // function attributes of that kernel, set before any stream capture (dfr_tile.cu)
 int prepare_volume_tile_dev(const Ctx& c);
 // the grid-size queries of the persistent volume kernels in that form, run

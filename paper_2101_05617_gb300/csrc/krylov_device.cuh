@@ -90,7 +90,7 @@ __device__ __forceinline__ double mgs_update_range_t(double* __restrict__ z, con
                                                      const double* __restrict__ VB, double h1, double h2, long long i,
                                                      long long i1, long long stride, const double* __restrict__ VC,
                                                      double h0, double acc = 0.0) {
-    constexpr int D = HC ? 4 : 8;   // entries in flight per thread
+  constexpr int D = HC ? 4 : 8;   // entries in flight per thread
   for (; i + (D - 1) * stride < i1; i += D * stride) {
     double v[D], b[D], a[D], c[D];
 #pragma unroll
@@ -138,10 +138,8 @@ __device__ __forceinline__ double mgs_update_range(double* __restrict__ z, const
                                                    const double* __restrict__ VB, double h1, double h2, long long i,
                                                    long long i1, long long stride,
                                                    const double* __restrict__ VC = nullptr, double h0 = 0.0) {
-  if (VC) {
-    return VA ? mgs_update_range_t<true, true>(z, VA, VB, h1, h2, i, i1, stride, VC, h0)
-              : mgs_update_range_t<false, true>(z, VA, VB, h1, h2, i, i1, stride, VC, h0);
-  }
+  // V_{j-2} only ever comes with V_{j-1}
+  if (VC) return mgs_update_range_t<true, true>(z, VA, VB, h1, h2, i, i1, stride, VC, h0);
   return VA ? mgs_update_range_t<true, false>(z, VA, VB, h1, h2, i, i1, stride, VC, h0)
             : mgs_update_range_t<false, false>(z, VA, VB, h1, h2, i, i1, stride, VC, h0);
 }
@@ -227,7 +225,6 @@ __device__ __forceinline__ double mgs_update_keep(double* __restrict__ z, const 
                                                   const double* __restrict__ VB, double h1, double h2, long long i0,
                                                   long long i1, long long stride, const double* __restrict__ VC,
                                                   double h0, double (&keep)[kKeep]) {
-  // V_{j-2} only ever comes with V_{j-1}
   if (VC) return mgs_update_keep_t<true, true>(z, VA, VB, h1, h2, i0, i1, stride, VC, h0, keep);
   return VA ? mgs_update_keep_t<true, false>(z, VA, VB, h1, h2, i0, i1, stride, VC, h0, keep)
             : mgs_update_keep_t<false, false>(z, VA, VB, h1, h2, i0, i1, stride, VC, h0, keep);
@@ -480,10 +477,7 @@ __device__ __forceinline__ int orth_dots_dev(const double* __restrict__ z, const
   double s[5];
   const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
   if (VC) {
-    if (VA)
-      orth_dots_range_t<true, true>(z, VB, VA, VC, i0, n, stride, s);
-    else
-      orth_dots_range_t<false, true>(z, VB, VA, VC, i0, n, stride, s);
+    orth_dots_range_t<true, true>(z, VB, VA, VC, i0, n, stride, s);
   } else if (VA) {
     orth_dots_range_t<true, false>(z, VB, VA, VC, i0, n, stride, s);
   } else {

@@ -111,8 +111,8 @@ struct Ctx {
   double* d_H = nullptr;
   double* d_F = nullptr;
   double* d_expm_ws = nullptr;    // expm workspace
-  double* d_partials = nullptr;   // reduction partials
-  double* d_vpart = nullptr;      // partials of the epilogue dot products (2 per volume block)
+  double* d_partials = nullptr;   // reduction partials, up to 5 per block (the complex64-bulk form's dots)
+  double* d_vpart = nullptr;      // partials of the epilogue dot products (3 or 5 per volume block)
   double* d_cdot = nullptr;       // V_j . V_{j-1} per basis index
   double* d_scal = nullptr;       // device scalars (see kiops.cu)
   // 0 happy flag, 1 happy size, 3 a bounded wait gave up, 8 ticket of the reductions and vector passes,
