@@ -798,7 +798,9 @@ int sw_jvp_linearized(sw_ctx_t c, const double* v, double* Jv, void* stream) {
     // the FP32 kernels read each entry of v several times: one FP32 copy (the
     // rounding they would do themselves, so the same result bit for bit)
     // instead of a conversion at every use.  6 x 60 x 60, p = 5: the product 54
-    // -> 36 us (its face kernel 29 -> 12 us)
+    // -> 36 us (its face kernel 29 -> 12 us); no smaller size measured pays for the
+    // third launch (C calls: 6 x 1 x 1, p = 3: 8.4 -> 8.2 us; 6 x 8 x 8: 10.4 -> 10.3;
+    // 6 x 16 x 16: 11.0 -> 10.3; 6 x 8 x 8, p = 5: 12.6 -> 10.3)
     if (int rc = launch_to_float(*c, v, c->d_v32, c->n, as_stream(stream))) return rc;
     ep.v32 = c->d_v32;
   }

@@ -59,7 +59,9 @@ __device__ __forceinline__ T load_state(const double* __restrict__ q, const doub
 // FP64 divisions and square roots are sequences of many FP64 instructions, so
 // each side takes a single reciprocal square root: with rs = 1 / sqrt(c q^0), c =
 // g_r h^dd / sqrt g, a^d = sqrt(c q^0) = c q^0 rs (corrected to the last bit by
-// one residual), 1 / a^d = rs and 1 / q^0 = c rs^2.
+// one residual), 1 / a^d = rs and 1 / q^0 = c rs^2 (some units in the last place off,
+// where a division is correctly rounded; the results' distance from a 64-bit
+// reference did not change).
 struct SpeedRoot {
   double a, ia, r;   // a^d, 1 / a^d, 1 / q^0
 };
@@ -68,7 +70,10 @@ __device__ __forceinline__ SpeedRoot speed_root(double q0, double c) {
   const double s = x * rs;
   return {fma(0.5 * rs, fma(-s, s, x), s), rs, c * rs * rs};
 }
-// a^d = sqrt(h^dd g_r H) (App. E) and the Froude number M = u^d / a^d
+// a^d = sqrt(h^dd g_r H) (App. E) and the Froude number M = u^d / a^d.  q^d (r ia) and
+// (q^d r) ia are equally accurate; which last bits they give decides accept/reject
+// choices of the window-2 phi solver at long steps (6 x 60 x 60, dt = 1800 s), and the
+// other one's choices led the benchmark's first start into a blown-up substep.
 __device__ __forceinline__ void speed_mach(double q0, double qd, double c, double& a, double& M) {
   const SpeedRoot z = speed_root(q0, c);
   a = z.a;

@@ -324,9 +324,11 @@ __device__ __forceinline__ void fx_sweep(const double (*sF)[3][NS * NS], const d
 // exponent EU = t + 2 - u and v^0 for EA = t + 2 - a puts all terms in one unit and
 // the fluxes come out as block values of exponent TF = t - 1020, t the largest of
 // a + e(v^0), u + e(v^i) and e(interface flux) + 1020 in the element (e: biased
-// exponents; the two spare bits are the sums' headroom).  The sources, stored
-// times -dx/2, add to the packed sweep shifted by k = De + u - s >= 0.  What is
-// left for the FP64 pipe is the conversion and scaling of three sums a node.
+// exponents; the two spare bits are the sums' headroom).  Both momentum components
+// share the exponent: the weaker one's fluxes hold fewer bits, by the ratio of the
+// two.  The sources, stored times -dx/2, add to the packed sweep shifted by k = De +
+// u - s >= 0.  What is left for the FP64 pipe is the conversion and scaling of three
+// sums a node.
 // 6 x 60 x 60, p = 5: 90 -> 81 us with the augmented operator and the dots, the
 // product with its face kernel 71 -> 67 us; 6 x 90 x 90, p = 6: 217 -> 188 us.
 struct LinExp {

@@ -353,7 +353,9 @@ __device__ __forceinline__ bool ens_task_ok(const EnsList& L, int lo, int ph, un
 
 // one Krylov iteration of every listed member (persistent, graph-captured);
 // 64 registers per thread at most (1024 threads per SM), as the single-grid
-// volume kernel
+// volume kernel; the three orders' bodies, each with its FP64 fallback, spill ~1 KB
+// there.  With the budget of 768 or 512 threads per SM an iteration took longer all
+// the same (235 and 291 us against 212 at the time)
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) ens_iter_kernel(const EnsDesc* __restrict__ desc, EnsDyn* __restrict__ dyn,
                                                          const EnsList* __restrict__ list, EnsCtl* ctl) {

@@ -11,10 +11,11 @@
 // h l' + l h' (l l' is below 2^-57 of the largest product).  The sums are exact
 // in 64 bits for up to twenty terms: |h|, |l| <= 2^29, so the h h' sum stays
 // below 20 2^58 < 2^63, and with the matrix' l' centred (|l'| <= 2^28) the
-// mixed sum below 20 (2^57 + 2^58) < 2^63.  Against the largest term the
-// result carries 58 bits where an FP64 chain rounds every partial sum to 53, so
-// the error is smaller than the FP64 chain's (measured against a 64-bit
-// reference; see the kernels).
+// mixed sum below 20 (2^57 + 2^58) < 2^63.  A block's largest value carries 58 bits
+// and the sum is rounded once, where an FP64 chain rounds every partial sum to 53:
+// against its largest terms a sum is more accurate (measured against a 64-bit
+// reference; see the kernels).  A value k bits below its block's largest one holds
+// 58 - k bits, so a sum of such values alone can hold fewer than an FP64 chain's.
 //
 // Blocks the format cannot hold faithfully -- a NaN, an infinity, a largest
 // magnitude outside 2^-623 .. 2^677 -- are left to the FP64 chain (fx_usable).
