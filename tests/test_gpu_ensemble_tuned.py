@@ -33,9 +33,9 @@ def test_tuned_is_not_slower(spec):
         return time.perf_counter() - t
 
     run()
-    untuned = min(run() for _ in range(4))
+    untuned = min(run() for _ in range(8))
     ens.tune(qs)
     run()
-    tuned = min(run() for _ in range(4))
+    tuned = min(run() for _ in range(8))
     ens.close()
     assert tuned < 1.08 * untuned, (tuned, untuned)
